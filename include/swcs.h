@@ -230,9 +230,10 @@ int swcs_probe_counts(swcs_ctx* ctx, int64_t* h_out4, int reset);
  *              beta-string space exceeds 2^22 or clusters cannot launch)
  *   "cluster"  CTAs per alpha-string row in the row sweep, 1..16 (default 1)
  *   "threads"  threads per CTA of the row sweep: 128, 256, 512 or 1024 (default 1024)
- *   "energy"   energy and sigma_D: 0 automatic (alpha-string rows when the
- *              sector allows, default), 1 probe kernel (connections of each D
- *              looked up in the state's index), 2 rows
+ *   "energy"   energy and sigma_D: 0 automatic (default: from the pairs of the
+ *              state's determinants at most two excitations apart), 1 probe
+ *              kernel (connections of each D looked up in the state's index),
+ *              2 alpha-string rows
  *   "row_occupancy" resident 512-thread CTAs per SM the row sweep is compiled
  *              for: 2 (default, 64 registers), 3 (40 registers) or 1 (no cap)
  *   "wait_timeout_ms"  bound of every device-side wait (default 2000)

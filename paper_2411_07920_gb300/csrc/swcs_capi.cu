@@ -13,6 +13,7 @@
 #include "../../include/swcs.h"
 #include "swcs_device.cuh"
 #include "swcs_kernels.h"
+#include "swcs_pairs.h"
 
 using namespace swcs;
 
@@ -83,6 +84,9 @@ struct swcs_ctx {
   int opt_screen_scatter = 1;  // a subset sweep marks and scatters only what the selected operators read
   bool screen_now = false;     // set around a subset sweep whose lists are built
 
+  // pairs of determinants (swcs_pairs.cu): string tables, grouped records, items
+  DevBuf pr_tab, pr_slot, pr_pos, pr_rec, pr_oth, pr_idx, pr_items;
+
   // external sigma table
   DevBuf ext;
   uint64_t ext_cap = 0;
@@ -117,6 +121,7 @@ struct Ctrl {
   unsigned long long ctr[12];
   long long stats[8];
   double acc[2];
+  PairCtl pairs;  // right after acc: one memset clears both
   double eout[2];
   unsigned long long n_distinct;
   double ovl[3];  // swcs_overlap: <state|given>, <given|given>, <state|state>
@@ -669,10 +674,61 @@ int sweep_rows(swcs_ctx* c, double* d_g, int64_t nd_bound = -1, bool enqueue = t
   return SWCS_OK;
 }
 
-// Energy (and optionally sigma_D in state order) through the row machinery;
-// 1 when not applicable.
+// Buffers and arguments of the pair enumeration for nd determinants; its tables and counters are reset here.
+int pair_args(swcs_ctx* c, int64_t nd, bool energy, PairArgs* out) {
+  Ctrl* k = ctrl(c);
+  const uint64_t tcap = pow2_at_least((uint64_t)std::max<int64_t>(2 * std::min<int64_t>(nd, c->NA), 64));
+  int r;
+  if ((r = ensure(c, c->pr_tab, 2 * tcap * sizeof(PairSlot))) || (r = ensure(c, c->pr_slot, (size_t)nd * 8)) ||
+      (r = ensure(c, c->pr_pos, (size_t)nd * 8)) || (r = ensure(c, c->pr_rec, (size_t)nd * 2 * sizeof(PairRec))) ||
+      (r = ensure(c, c->pr_oth, (size_t)nd * 8)) || (r = ensure(c, c->pr_items, (size_t)nd * 2 * sizeof(uint4))) ||
+      (energy && (r = ensure(c, c->pr_idx, (size_t)nd * 8))))
+    return r;
+  PairArgs a{};
+  a.H = ham_dev(c);
+  a.m = c->n / 2;
+  a.keys = (const uint64_t*)c->keys_a.p;
+  a.amps = (const double*)c->amps_a.p;
+  a.n = &k->n_state;
+  a.cap = (uint32_t)nd;
+  a.tab = (PairSlot*)c->pr_tab.p;
+  a.mask = (uint32_t)(tcap - 1);
+  a.slot_of = (uint32_t*)c->pr_slot.p;
+  a.pos_of = (uint32_t*)c->pr_pos.p;
+  a.rec = (PairRec*)c->pr_rec.p;
+  a.oth = (uint32_t*)c->pr_oth.p;
+  a.idx = (uint32_t*)c->pr_idx.p;
+  a.items = (uint4*)c->pr_items.p;
+  a.blk = nd <= 65536 ? 4 : nd <= 262144 ? 8 : 32;  // enough items for every warp of the device
+  a.ctl = &k->pairs;
+  a.acc = k->acc;
+  a.err = &k->err;
+  CK(cudaMemsetAsync(c->pr_tab.p, 0xff, 2 * tcap * sizeof(PairSlot), c->st));
+  CK(cudaMemsetAsync(k->acc, 0, sizeof(k->acc) + sizeof(PairCtl), c->st));
+  *out = a;
+  return SWCS_OK;
+}
+
+constexpr int64_t kMaxPairDets = (int64_t)1 << 27;  // places of determinants share a word with five more bits
+
+// Energy (and optionally sigma_D in state order): from the pairs of determinants of the state, or through the
+// row machinery where that was asked for (option "energy" 2) or hash probes are to be counted; 1 when neither applies.
 int energy_rows(swcs_ctx* c, double* sig_out) {
   if (c->opt_energy == 1) return 1;
+  if (c->opt_energy == 0 && !c->opt_count_probes) {
+    const int64_t nd = host_state_size(c);
+    if (nd < 0) return fail(c, SWCS_ERR_CUDA, "cannot read state size");
+    if (nd <= kMaxPairDets) {
+      PairArgs a;
+      const int r = pair_args(c, nd, true, &a);
+      if (r) return r;
+      a.sig = sig_out;
+      CK(launch_k(c, kKEnergy, [&] { return launch_pairs_energy(a, nd, c->nsm, c->st); }));
+      c->launches += 3;
+      CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(ctrl(c)->acc, ctrl(c)->eout, c->st); }));
+      return SWCS_OK;
+    }
+  }
   return sweep_rows(c, nullptr, -1, true, nullptr, true, sig_out);
 }
 
@@ -819,7 +875,7 @@ int swcs_destroy(swcs_ctx* c) {
                     &c->ck_keys, &c->ck_amps, &c->ck_n, &c->sn_keys, &c->sn_amps, &c->sn_n, &c->sigma, &c->nu0,
                     &c->nu1, &c->atab0, &c->atab1, &c->dth, &c->pool_dev, &c->selbits, &c->feat,
                     &c->ypred, &c->topk_hist, &c->topk_ctl, &c->occ, &c->prb, &c->ab_cnt, &c->ab_list,
-                    &c->selhist};
+                    &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items};
   for (DevBuf* b : bufs) release(*b);
   if (c->pin) cudaFreeHost(c->pin);
   for (auto& e : c->ev_pending) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }

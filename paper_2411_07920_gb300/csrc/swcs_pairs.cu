@@ -1,0 +1,565 @@
+// Pairs of determinants of the state that differ by at most two or three
+// excitations, found without visiting the external space, and what is summed
+// over them: the energy and sigma_D on the state (two-body operators connect
+// ranks 0..2), and the state's three-body density matrices (ranks 0..3).
+//
+// A pair (D, D') of rank (d_alpha, d_beta) with d_alpha + d_beta <= 3 has
+// min(d_alpha, d_beta) <= 1.  So the state is grouped twice, by alpha string
+// and by beta string, and each side only joins a group with itself and with
+// the groups whose string is ONE single excitation away (no * nv hash lookups
+// per string); inside a pair of groups the other spin's strings are compared
+// by XOR and population count.  The alpha side counts the pairs with
+// d_alpha <= 1, the beta side those with d_beta <= 1 and d_alpha >= 2, so each
+// pair is met once.  At 52 spin-orbitals, 12 electrons and 10^6 determinants
+// that is about 2e9 comparisons for 1.7e8 pairs, where the sweeps over
+// connected determinants walk 2e10 pairs.  Energy and sigma_D there: 2.1 ms
+// (65.2 ms by alpha-string rows); 0.05 ms for 257 determinants (1.8 ms: the
+// rows visit every alpha string of the sector), 0.22 ms at 28/8 with 38,701
+// (0.86 ms).  Bound by L2: table lookups, the integrals and the additions.
+//
+// One warp takes one item: up to 32 determinants of a group against the
+// concatenated determinants of the group and its neighbours, 32 at a time (a
+// lane holds one of them; the loop runs over the item's determinants).  Hits
+// go to queues in shared memory, by rank, and are worked off 32 at a time, so
+// the long path per hit runs on full, converged warps however rare hits are.
+//
+// Signs: amplitudes are held in the spin-blocked convention, |D> = (alpha
+// creators in order)(beta creators in order)|0>, where the phase of a
+// spin-conserving operator factors into the two strings: the parity of
+// occupied orbitals below t is bit t of a prefix-XOR of the string, so the
+// phase of removing a set T is the parity of (prefix & T).  The conversion to
+// the interleaved convention of the state is one sign per determinant.
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "swcs_device.cuh"
+#include "swcs_kernels.h"
+#include "swcs_pairs.h"
+
+namespace swcs {
+
+namespace {
+
+constexpr int kPairThreads = 256;
+constexpr int kPairWarps = kPairThreads / 32;
+constexpr int kMaxSeg = 1 + 256;  // the group itself and its single-excitation neighbours (no * nv <= 256)
+constexpr uint32_t kNoString = 0xFFFFFFFFu;
+
+__device__ __forceinline__ uint32_t even32(uint64_t x) {
+  x &= 0x5555555555555555ull;
+  x = (x | (x >> 1)) & 0x3333333333333333ull;
+  x = (x | (x >> 2)) & 0x0F0F0F0F0F0F0F0Full;
+  x = (x | (x >> 4)) & 0x00FF00FF00FF00FFull;
+  x = (x | (x >> 8)) & 0x0000FFFF0000FFFFull;
+  x = (x | (x >> 16)) & 0x00000000FFFFFFFFull;
+  return (uint32_t)x;
+}
+
+// Bit t: parity of the occupied orbitals below t.
+__device__ __forceinline__ uint32_t below_parity(uint32_t x) {
+  x ^= x << 1;
+  x ^= x << 2;
+  x ^= x << 4;
+  x ^= x << 8;
+  x ^= x << 16;
+  return x << 1;
+}
+
+__device__ __forceinline__ int parity32(uint32_t x) { return __popc(x) & 1; }
+
+// Sign between the interleaved and the spin-blocked order of D's creators: pairs (alpha a, beta b) with b < a.
+__device__ __forceinline__ int blocked_sign(uint32_t xa, uint32_t xb) { return parity32(below_parity(xb) & xa); }
+
+// Phase bit of the single a+_r a_p on string x.
+__device__ __forceinline__ int single_sign(uint32_t x, int p, int r) {
+  const int lo = min(p, r), hi = max(p, r);
+  const uint32_t between = ((1u << hi) - 1u) & ~((2u << lo) - 1u);
+  return parity32(x & between);
+}
+
+__device__ __forceinline__ uint32_t string_slot(uint32_t key, uint32_t mask) { return (uint32_t)mix64(key) & mask; }
+
+// ---------------------------------------------------------------- grouping by string, both spins
+__global__ void pair_insert_kernel(PairArgs A) {
+  const long long n = *A.n;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * n; t += (long long)gridDim.x * blockDim.x) {
+    const int s = t >= n;
+    const long long i = t - (s ? n : 0);
+    const uint32_t key = even32(A.keys[i] >> s);
+    PairSlot* tab = A.tab + (s ? (size_t)A.mask + 1 : 0);
+    uint32_t at = string_slot(key, A.mask);
+    bool found = false;
+    for (uint32_t k = 0; k <= A.mask; ++k) {
+      uint32_t prev = *(volatile uint32_t*)&tab[at].key;
+      if (prev == kNoString) prev = atomicCAS(&tab[at].key, kNoString, key);
+      if (prev == kNoString || prev == key) {
+        found = true;
+        break;
+      }
+      at = (at + 1) & A.mask;
+    }
+    if (!found) {
+      set_error(A.err, kDevTableFull);
+      at = 0;
+    }
+    A.slot_of[t] = at;
+    A.pos_of[t] = atomicAdd(&tab[at].cnt, 1u) + 1u;  // counters start at -1
+  }
+}
+
+// Ranges of the groups in the grouped order (any order: one atomic per warp) and the items, blk determinants each.
+__global__ void pair_alloc_kernel(PairArgs A) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t cap = A.mask + 1;
+  for (uint32_t t0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; t0 < 2 * cap; t0 += gridDim.x * blockDim.x) {
+    const uint32_t t = t0 + lane;  // tables have at least 64 slots: a warp stays inside one of them
+    const int s = t0 >= cap;
+    PairSlot sl = A.tab[t];
+    const uint32_t c = sl.key == kNoString ? 0u : sl.cnt + 1u;
+    const uint32_t it = (c + A.blk - 1u) / A.blk;
+    unsigned long long v = ((unsigned long long)it << 32) | c, inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    unsigned long long base = 0;
+    const unsigned long long tot = __shfl_sync(0xffffffffu, inc, 31);
+    if (tot == 0) continue;
+    if (lane == 0) base = atomicAdd(&A.ctl->alloc[s], tot);
+    base = __shfl_sync(0xffffffffu, base, 0) + inc - v;
+    if (!c) continue;
+    const uint32_t off = (uint32_t)base;
+    A.tab[t].off = off;
+    uint4* items = A.items + (s ? A.cap : 0) + (uint32_t)(base >> 32);
+    for (uint32_t b = 0; b < it; ++b) items[b] = make_uint4(sl.key, off, c, b);
+  }
+}
+
+__device__ __forceinline__ double diagonal_element(const HamDev& H, uint64_t d) {
+  double e = 0.0;
+  for (uint64_t x = d; x; x &= x - 1ull) {
+    const int a = __ffsll((long long)x) - 1;
+    double j = 0.0;
+    for (uint64_t y = d; y; y &= y - 1ull) j += __ldg(&H.J[a * H.n + __ffsll((long long)y) - 1]);
+    e += __ldg(&H.h[a * H.n + a]) + 0.5 * j;
+  }
+  return e;
+}
+
+// Records in grouped order, <psi|psi>; with ENERGY the diagonal part of sigma and of the energy.
+template <bool ENERGY>
+__global__ void pair_records_kernel(PairArgs A) {
+  __shared__ double red[2][kPairWarps];
+  const long long n = *A.n;
+  double s2 = 0.0, e = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const uint64_t d = A.keys[i];
+    const double c = A.amps[i];
+    const uint32_t xa = even32(d), xb = even32(d >> 1);
+    const uint32_t neg = (uint32_t)blocked_sign(xa, xb);
+    const double cb = neg ? -c : c;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const size_t t = (size_t)i + (s ? (size_t)n : 0);
+      const uint32_t slot = A.slot_of[t];
+      const size_t pos = (size_t)(s ? A.cap : 0) + A.tab[slot + (s ? A.mask + 1 : 0)].off + A.pos_of[t];
+      PairRec r;
+      r.own = s ? xb : xa;
+      r.oth = s ? xa : xb;
+      r.amp = cb;
+      A.rec[pos] = r;
+      A.oth[pos] = r.oth;
+      if (ENERGY) A.idx[pos] = (uint32_t)i | (neg << 31);
+    }
+    s2 += c * c;
+    if (ENERGY) {
+      const double sg = diagonal_element(A.H, d) * c;
+      e += c * sg;
+      if (A.sig) A.sig[i] = sg;
+    }
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    e += __shfl_xor_sync(0xffffffffu, e, o);
+  }
+  if (lane == 0) {
+    red[0][warp] = s2;
+    red[1][warp] = e;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double t = 0.0;
+    for (int w = 0; w < kPairWarps; ++w) t += red[threadIdx.x][w];
+    if (t != 0.0) atomicAdd(&A.acc[1 - threadIdx.x], t);
+  }
+}
+
+// ---------------------------------------------------------------- what a pair adds
+// <D'|H|D> in the spin-blocked convention, D -> D' of rank 1 or 2.
+__device__ __forceinline__ double pair_element(const HamDev& H, int s, const PairRec& a, const PairRec& b) {
+  const uint32_t xs = a.own ^ b.own, xo = a.oth ^ b.oth;
+  const int n = H.n, o = 1 - s;
+  const uint32_t rs = xs & a.own, as = xs & b.own, ro = xo & a.oth, ao = xo & b.oth;
+  if (__popc(xs) + __popc(xo) == 2) {
+    const int sp = xs ? s : o;
+    const uint32_t str = xs ? a.own : a.oth;
+    const int p = __ffs(xs ? rs : ro) - 1, r = __ffs(xs ? as : ao) - 1;
+    const int P = 2 * p + sp, R = 2 * r + sp;
+    double f = __ldg(&H.h[R * n + P]);
+    const double* w = H.Ws + ((size_t)P * n + R) * n;
+    for (uint32_t x = a.own; x; x &= x - 1u) f += __ldg(&w[2 * (__ffs(x) - 1) + s]);
+    for (uint32_t x = a.oth; x; x &= x - 1u) f += __ldg(&w[2 * (__ffs(x) - 1) + o]);
+    return apply_sign(f, single_sign(str, p, r));
+  }
+  if (xs && xo) {  // one excitation of each spin
+    const int p = __ffs(rs) - 1, r = __ffs(as) - 1, i = __ffs(ro) - 1, j = __ffs(ao) - 1;
+    const int P = 2 * p + s, R = 2 * r + s, I = 2 * i + o, J = 2 * j + o;
+    const int sb = single_sign(a.own, p, r) ^ single_sign(a.oth, i, j) ^ (int)(P > I) ^ (int)(R > J);
+    const double g = __ldg(&H.G[(size_t)pair_index(min(P, I), max(P, I), n) * H.npairs + pair_index(min(R, J), max(R, J), n)]);
+    return apply_sign(g, sb);
+  }
+  const int sp = xs ? s : o;
+  const uint32_t str = xs ? a.own : a.oth, rm = xs ? rs : ro, ad = xs ? as : ao;
+  const int p = __ffs(rm) - 1, q = 31 - __clz(rm), r = __ffs(ad) - 1, t = 31 - __clz(ad);
+  // a+_r a+_t a_q a_p: (below p) + (below q without p) + (below t in the rest) + (below r in the rest with t)
+  const uint32_t mid = str & ~rm;
+  const uint32_t pa = below_parity(str), pm = below_parity(mid);
+  const int sb = parity32(pa & rm) ^ parity32(pm & ad) ^ 1;  // the p below q counts once; r lies below t
+  const double g = __ldg(&H.G[(size_t)pair_index(2 * p + sp, 2 * q + sp, n) * H.npairs + pair_index(2 * r + sp, 2 * t + sp, n)]);
+  return apply_sign(g, sb);
+}
+
+__device__ __forceinline__ uint32_t pair_of(uint32_t two) {  // index of the pair of set bits
+  const uint32_t a = __ffs(two) - 1, b = 31 - __clz(two);
+  return b * (b - 1) / 2 + a;
+}
+
+__device__ __forceinline__ uint32_t triple_of(uint32_t three) {
+  const uint32_t a = __ffs(three) - 1, c = 31 - __clz(three);
+  const uint32_t b = __ffs(three & (three - 1u)) - 1;
+  return c * (c - 1) * (c - 2) / 6 + b * (b - 1) / 2 + a;
+}
+
+// Both determinants of a pair with the prefix parities of their strings (index 0: own spin s, 1: the other).
+struct PairStrings {
+  uint32_t xi[2], xj[2], pi[2], pj[2];
+  double cc;
+};
+
+// Gamma(T, T') of the mixed block whose pair has the spin of string k: pair masks Pi -> Pj, single Si -> Sj of
+// the other string; only the upper triangle is kept.
+__device__ __forceinline__ void add_mixed(const PairArgs& A, int s, int k, const PairStrings& P, uint32_t Pi, uint32_t Pj,
+                                          uint32_t Si, uint32_t Sj) {
+  const uint32_t par = (P.pi[k] & Pi) ^ (P.pj[k] & Pj);
+  const uint32_t par2 = (P.pi[1 - k] & Si) ^ (P.pj[1 - k] & Sj);
+  const int sb = (__popc(par) + __popc(par2)) & 1;
+  const uint32_t np = A.m * (A.m - 1) / 2;
+  const uint32_t T = (__ffs(Si) - 1) * np + pair_of(Pi), U = (__ffs(Sj) - 1) * np + pair_of(Pj);
+  double* M = A.mix[s ^ k];
+  atomicAdd(&M[(size_t)min(T, U) * A.ld_mix + max(T, U)], apply_sign(P.cc, sb));
+}
+
+__device__ __forceinline__ void add_same(const PairArgs& A, int s, int k, const PairStrings& P, uint32_t Ti, uint32_t Tj) {
+  const int sb = parity32((P.pi[k] & Ti) ^ (P.pj[k] & Tj));
+  const uint32_t T = triple_of(Ti), U = triple_of(Tj);
+  double* M = A.same[s ^ k];
+  atomicAdd(&M[(size_t)min(T, U) * A.ld_same + max(T, U)], apply_sign(P.cc, sb));
+}
+
+__device__ __forceinline__ PairStrings pair_strings(const PairRec& a, const PairRec& b, uint32_t rm[2], uint32_t ad[2],
+                                                    uint32_t cm[2]) {
+  PairStrings P;
+  P.xi[0] = a.own; P.xi[1] = a.oth; P.xj[0] = b.own; P.xj[1] = b.oth;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    P.pi[k] = below_parity(P.xi[k]);
+    P.pj[k] = below_parity(P.xj[k]);
+    const uint32_t x = P.xi[k] ^ P.xj[k];
+    rm[k] = x & P.xi[k];
+    ad[k] = x & P.xj[k];
+    cm[k] = P.xi[k] & P.xj[k];
+  }
+  P.cc = a.amp * b.amp;
+  return P;
+}
+
+// Rank 3: one element.
+__device__ __forceinline__ void add_rank3(const PairArgs& A, int s, const PairRec& a, const PairRec& b) {
+  uint32_t rm[2], ad[2], cm[2];
+  const PairStrings P = pair_strings(a, b, rm, ad, cm);
+  if (rm[0] == 0) add_same(A, s, 1, P, rm[1], ad[1]);
+  else add_mixed(A, s, 1, P, rm[1], ad[1], rm[0], ad[0]);  // one own excitation, two of the other spin, on either side
+}
+
+// Rank 2: an element for each spectator orbital common to both determinants.
+__device__ __forceinline__ void add_rank2(const PairArgs& A, int s, const PairRec& a, const PairRec& b) {
+  uint32_t rm[2], ad[2], cm[2];
+  const PairStrings P = pair_strings(a, b, rm, ad, cm);
+  const bool one_each = rm[0] != 0;
+  for (uint32_t x = cm[0]; x; x &= x - 1u) {
+    const uint32_t t = x & (0u - x);
+    if (one_each) add_mixed(A, s, 0, P, rm[0] | t, ad[0] | t, rm[1], ad[1]);
+    else add_mixed(A, s, 1, P, rm[1], ad[1], t, t);
+  }
+  for (uint32_t x = cm[1]; x; x &= x - 1u) {
+    const uint32_t t = x & (0u - x);
+    if (one_each) add_mixed(A, s, 1, P, rm[1] | t, ad[1] | t, rm[0], ad[0]);
+    else add_same(A, s, 1, P, rm[1] | t, ad[1] | t);
+  }
+}
+
+// Rank 1, by the whole warp: an element for each pair of spectators, lanes over the pairs.
+__device__ __forceinline__ void add_rank1(const PairArgs& A, int s, const PairRec& a, const PairRec& b, int lane) {
+  uint32_t rm[2], ad[2], cm[2];
+  const PairStrings P = pair_strings(a, b, rm, ad, cm);
+  const int k = rm[0] ? 0 : 1;  // the string that changes
+  const int n0 = __popc(cm[k]), n1 = __popc(cm[1 - k]), nc = n0 + n1;
+  for (int c = lane; c < nc * (nc - 1) / 2; c += 32) {
+    int y = (int)((1.0f + sqrtf(8.0f * (float)c + 1.0f)) * 0.5f);
+    while (y * (y - 1) / 2 > c) --y;
+    while ((y + 1) * y / 2 <= c) ++y;
+    const int x = c - y * (y - 1) / 2;  // spectators x < y; the first n0 are of the changing string
+    const uint32_t t = 1u << (x < n0 ? __fns(cm[k], 0, x + 1) : __fns(cm[1 - k], 0, x - n0 + 1));
+    const uint32_t u = 1u << (y < n0 ? __fns(cm[k], 0, y + 1) : __fns(cm[1 - k], 0, y - n0 + 1));
+    if (y < n0) add_same(A, s, k, P, rm[k] | t | u, ad[k] | t | u);
+    else if (x < n0) add_mixed(A, s, k, P, rm[k] | t, ad[k] | t, u, u);
+    else add_mixed(A, s, 1 - k, P, t | u, t | u, rm[k], ad[k]);
+  }
+}
+
+// ---------------------------------------------------------------- the pairs
+template <bool ENERGY>
+__global__ void __launch_bounds__(kPairThreads) pair_kernel(PairArgs A) {
+  __shared__ uint32_t s_off[kPairWarps][kMaxSeg], s_pre[kPairWarps][kMaxSeg];
+  __shared__ uint32_t s_queue[kPairWarps][ENERGY ? 1 : 2][64];
+  __shared__ PairRec s_rec[kPairWarps][32];
+  __shared__ uint8_t s_occ[kPairWarps][32], s_vir[kPairWarps][32];
+  __shared__ double red[kPairWarps];
+  constexpr int R = ENERGY ? 2 : 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t n_it0 = (uint32_t)(A.ctl->alloc[0] >> 32), n_it1 = (uint32_t)(A.ctl->alloc[1] >> 32);
+  const int m = A.m, no = A.H.no, nv = A.H.nv;
+  double e_acc = 0.0;
+  for (;;) {
+    uint32_t w = 0;
+    if (lane == 0) w = atomicAdd(&A.ctl->next, 1u);
+    w = __shfl_sync(0xffffffffu, w, 0);
+    if (w >= n_it0 + n_it1) break;
+    const int s = w >= n_it0;
+    const uint4 item = A.items[(s ? A.cap : 0) + w - (s ? n_it0 : 0)];
+    const uint32_t str = item.x;
+    const PairRec* rec = A.rec + (s ? A.cap : 0);
+    const uint32_t* oth = A.oth + (s ? A.cap : 0);
+    const uint32_t i0 = item.y + item.w * A.blk;
+    const int ni = (int)min(A.blk, item.z - item.w * A.blk);
+    __syncwarp();
+    if (lane < ni) s_rec[warp][lane] = rec[i0 + lane];
+    // segments: the group itself from this item's determinants on, then the neighbours with a larger string
+    uint32_t tot = item.z - item.w * A.blk;
+    int nseg = 1;
+    if (lane == 0) {
+      s_off[warp][0] = i0;
+      s_pre[warp][0] = 0;
+    }
+    if (s == 0 || !ENERGY) {
+      const bool inr = lane < m, occ = inr && ((str >> lane) & 1u);
+      const unsigned bo = __ballot_sync(0xffffffffu, occ), bv = __ballot_sync(0xffffffffu, inr && !occ);
+      const unsigned lt = (1u << lane) - 1u;
+      if (occ) s_occ[warp][__popc(bo & lt)] = (uint8_t)lane;
+      else if (inr) s_vir[warp][__popc(bv & lt)] = (uint8_t)lane;
+      __syncwarp();
+      const PairSlot* tab = A.tab + (s ? (size_t)A.mask + 1 : 0);
+      for (int c0 = 0; c0 < no * nv; c0 += 32) {
+        const int c = c0 + lane;
+        uint32_t off = 0, cnt = 0;
+        if (c < no * nv) {
+          const uint32_t nb = str ^ (1u << s_occ[warp][c / nv]) ^ (1u << s_vir[warp][c % nv]);
+          if (nb > str) {
+            uint32_t at = string_slot(nb, A.mask);
+            for (uint32_t k = 0; k <= A.mask; ++k) {
+              const uint4 sl = __ldg((const uint4*)&tab[at]);
+              if (sl.x == nb) {
+                cnt = sl.y + 1u;
+                off = sl.z;
+                break;
+              }
+              if (sl.x == kNoString) break;
+              at = (at + 1) & A.mask;
+            }
+          }
+        }
+        const unsigned f = __ballot_sync(0xffffffffu, cnt > 0);
+        uint32_t inc = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += u;
+        }
+        if (cnt) {
+          const int k = nseg + __popc(f & lt);
+          s_off[warp][k] = off;
+          s_pre[warp][k] = tot + inc - cnt;
+        }
+        nseg += __popc(f);
+        tot += __shfl_sync(0xffffffffu, inc, 31);
+      }
+    }
+    __syncwarp();
+      int qn[2] = {0, 0}, seg = 0;
+    // works off the first cnt hits of a queue: the energy's, or those of rank 3 (0) and of rank 2 (1)
+    auto flush = [&](int which, int cnt) {
+      __syncwarp();
+      if (lane < cnt) {
+        const uint32_t q = s_queue[warp][which][lane];
+        const int i = (int)(q & 31u);
+        const uint32_t j = q >> 5;
+        const PairRec a = s_rec[warp][i], b = rec[j];
+        if (ENERGY) {
+          const double v = pair_element(A.H, s, a, b);
+          e_acc += 2.0 * v * a.amp * b.amp;
+          if (A.sig) {
+            const uint32_t* idx = A.idx + (s ? A.cap : 0);
+            const uint32_t ti = idx[i0 + i], tj = idx[j];
+            atomicAdd(&A.sig[ti & 0x7FFFFFFFu], apply_sign(v * b.amp, (int)(ti >> 31)));
+            atomicAdd(&A.sig[tj & 0x7FFFFFFFu], apply_sign(v * a.amp, (int)(tj >> 31)));
+          }
+        } else if (which == 0) {
+          add_rank3(A, s, a, b);
+        } else {
+          add_rank2(A, s, a, b);
+        }
+      }
+      __syncwarp();
+    };
+    auto push = [&](int which, bool hit, uint32_t code) {
+      const unsigned bal = __ballot_sync(0xffffffffu, hit);
+      if (!bal) return;
+      if (hit) s_queue[warp][which][qn[which] + __popc(bal & ((1u << lane) - 1u))] = code;
+      qn[which] += __popc(bal);
+      if (qn[which] >= 32) {
+        flush(which, 32);
+        qn[which] -= 32;
+        if (lane < qn[which]) s_queue[warp][which][lane] = s_queue[warp][which][32 + lane];
+        __syncwarp();
+      }
+    };
+    for (uint32_t f0 = 0; f0 < tot; f0 += 32) {
+      const uint32_t f = f0 + lane;
+      const bool live = f < tot;
+      while (live && seg + 1 < nseg && s_pre[warp][seg + 1] <= f) ++seg;
+      const uint32_t j = live ? s_off[warp][seg] + (f - s_pre[warp][seg]) : 0u;
+      const uint32_t bj = live ? __ldg(&oth[j]) : 0u;
+      const int d = seg > 0 ? 1 : 0;
+      // accepted ranks of the other spin, as set bits of the XOR; a beta-side pair has alpha rank >= 2
+      const int hi = live ? 2 * (R - d) : -1, lo = s ? 4 : (d ? 0 : 2);
+      const int before = d ? 32 : (int)min(32u, f);  // own group: determinants ahead of this one (f = its place from i0 on)
+      for (int i = 0; i < ni; ++i) {
+        const int pc = __popc(bj ^ s_rec[warp][i].oth);
+        const bool hit = pc <= hi && pc >= lo && i < before;
+        if (!__any_sync(0xffffffffu, hit)) continue;
+        const uint32_t code = (j << 5) | (uint32_t)i;
+        if (ENERGY) {
+          push(0, hit, code);
+        } else {
+          const int rank = d + (pc >> 1);
+          push(0, hit && rank == 3, code);
+          push(1, hit && rank == 2, code);
+          for (unsigned b1 = __ballot_sync(0xffffffffu, hit && rank == 1); b1; b1 &= b1 - 1u) {
+            const uint32_t jj = __shfl_sync(0xffffffffu, j, __ffs(b1) - 1);
+            add_rank1(A, s, s_rec[warp][i], rec[jj], lane);
+          }
+        }
+      }
+    }
+    flush(0, qn[0]);
+    if (!ENERGY) flush(1, qn[1]);
+  }
+  if (ENERGY) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e_acc += __shfl_xor_sync(0xffffffffu, e_acc, o);
+    if (lane == 0) red[warp] = e_acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int k = 0; k < kPairWarps; ++k) t += red[k];
+      if (t != 0.0) atomicAdd(&A.acc[0], t);
+    }
+  }
+}
+
+// Diagonal of the three-body matrices: Gamma(T, T) = sum of c_D^2 over the D that hold T.  One warp per item of
+// the grouping: the determinants of an item share the string X, so their weights are first summed per orbital of
+// the other spin (lane = orbital) and each pair of X then takes one addition per such orbital, each triple of X
+// one (per determinant it would be C(n_e, 3) additions, most of them to the few orbitals every determinant holds).
+__global__ void __launch_bounds__(kPairThreads) gamma_diagonal_kernel(PairArgs A) {
+  __shared__ uint8_t s_o[kPairWarps][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, no = A.H.no, np = no * (no - 1) / 2;
+  const uint32_t n_it0 = (uint32_t)(A.ctl->alloc[0] >> 32), n_it1 = (uint32_t)(A.ctl->alloc[1] >> 32);
+  for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < n_it0 + n_it1; w += (gridDim.x * blockDim.x) >> 5) {
+    const int s = w >= n_it0;
+    const uint4 item = A.items[(s ? A.cap : 0) + w - (s ? n_it0 : 0)];
+    const PairRec* rec = A.rec + (s ? A.cap : 0) + item.y + item.w * A.blk;
+    const int ni = (int)min(A.blk, item.z - item.w * A.blk);
+    PairRec r;
+    r.oth = 0;
+    r.amp = 0.0;
+    if (lane < ni) r = rec[lane];
+    double total = 0.0, mine = 0.0;  // all determinants' weight, and that of those holding orbital `lane`
+    for (int i = 0; i < ni; ++i) {
+      const double c = __shfl_sync(0xffffffffu, r.amp, i);
+      const uint32_t o = __shfl_sync(0xffffffffu, r.oth, i);
+      total += c * c;
+      if ((o >> lane) & 1u) mine += c * c;
+    }
+    __syncwarp();
+    if ((item.x >> lane) & 1u) s_o[warp][__popc(item.x & ((1u << lane) - 1u))] = (uint8_t)lane;
+    __syncwarp();
+    int x1 = 0, x2 = 1;
+    for (int t = 0; t < np; ++t) {
+      const size_t a = s_o[warp][x1], b = s_o[warp][x2];
+      const size_t T = b * (b - 1) / 2 + a;
+      if (mine != 0.0) {
+        const size_t q = (size_t)lane * (A.m * (A.m - 1) / 2) + T;
+        atomicAdd(&A.mix[s][q * A.ld_mix + q], mine);
+      }
+      for (int y = x2 + 1 + lane; y < no; y += 32) {
+        const size_t c = s_o[warp][y];
+        const size_t q = c * (c - 1) * (c - 2) / 6 + T;
+        atomicAdd(&A.same[s][q * A.ld_same + q], total);
+      }
+      if (++x1 == x2) {
+        x1 = 0;
+        ++x2;
+      }
+    }
+  }
+}
+
+}  // namespace
+
+// Grouped records of the state for both spins; A.tab filled with 0xff, A.ctl and A.acc zeroed before.
+cudaError_t launch_pairs_energy(const PairArgs& a, int64_t n, int nsm, cudaStream_t st) {
+  const int nb = (int)((2 * n + 255) / 256 < 8 * nsm ? (2 * n + 255) / 256 : 8 * nsm);
+  const int tb = (int)((2 * ((int64_t)a.mask + 1) + 255) / 256 < 8 * nsm ? (2 * ((int64_t)a.mask + 1) + 255) / 256 : 8 * nsm);
+  pair_insert_kernel<<<nb, 256, 0, st>>>(a);
+  pair_alloc_kernel<<<tb, 256, 0, st>>>(a);
+  pair_records_kernel<true><<<nb, kPairThreads, 0, st>>>(a);
+  pair_kernel<true><<<4 * nsm, kPairThreads, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pairs_gamma(const PairArgs& a, int64_t n, int nsm, cudaStream_t st) {
+  const int nb = (int)((2 * n + 255) / 256 < 8 * nsm ? (2 * n + 255) / 256 : 8 * nsm);
+  const int tb = (int)((2 * ((int64_t)a.mask + 1) + 255) / 256 < 8 * nsm ? (2 * ((int64_t)a.mask + 1) + 255) / 256 : 8 * nsm);
+  pair_insert_kernel<<<nb, 256, 0, st>>>(a);
+  pair_alloc_kernel<<<tb, 256, 0, st>>>(a);
+  pair_records_kernel<false><<<nb, kPairThreads, 0, st>>>(a);
+  pair_kernel<false><<<4 * nsm, kPairThreads, 0, st>>>(a);
+  gamma_diagonal_kernel<<<8 * nsm, kPairThreads, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace swcs
