@@ -144,8 +144,9 @@ int swcs_energy_dev(swcs_ctx* ctx, double* d_out);
 /* Pool gradient g_k = 2 <psi|H A_k|psi>/<psi|psi>, A_k = tau_k - tau_k^dag,
  * for the canonical pool (ADAPT step 4, Sec. II.C).  h_subset == NULL:
  * all pool entries are written to h_g_out[pool_size]; otherwise only
- * h_g_out[h_subset[i]] for i < n_subset (other entries untouched).  With a
- * subset the device variant's alpha-string row sweep first marks, for each
+ * h_g_out[h_subset[i]] for i < n_subset (other entries untouched).  From
+ * density matrices (option "pairs") the whole gradient is formed either way.
+ * With a subset the device variant's alpha-string row sweep first marks, for each
  * target alpha string, the row sectors that the selected operators read (and
  * those of the state's own determinants, so the energy stays exact), forms
  * sigma only there -- every other connected pair is skipped before its
@@ -225,7 +226,7 @@ int swcs_stats(swcs_ctx* ctx, int64_t* h_out8);
 int swcs_probe_counts(swcs_ctx* ctx, int64_t* h_out4, int reset);
 
 /* Tuning options (no effect on results beyond FP64 summation order):
- *   "sweep"    0 automatic (default), 1 hashed external-sigma table,
+ *   "sweep"    0 automatic (default; see "pairs"), 1 hashed external-sigma table,
  *              2 alpha-string rows (SWCS_ERR_INVALID_ARG when the sector's
  *              beta-string space exceeds 2^22 or clusters cannot launch)
  *   "cluster"  CTAs per alpha-string row in the row sweep, 1..16 (default 1)
@@ -234,6 +235,11 @@ int swcs_probe_counts(swcs_ctx* ctx, int64_t* h_out4, int reset);
  *              state's determinants at most two excitations apart), 1 probe
  *              kernel (connections of each D looked up in the state's index),
  *              2 alpha-string rows
+ *   "pairs"    automatic pool sweep ("sweep" 0) from the state's density
+ *              matrices instead of alpha-string rows: -1 (default) where the
+ *              state is sparse enough for it to be faster, 0 never, 1 wherever
+ *              it applies (at least two electrons of each spin, no counting of
+ *              hash probes)
  *   "row_occupancy" resident 512-thread CTAs per SM the row sweep is compiled
  *              for: 2 (default, 64 registers), 3 (40 registers) or 1 (no cap)
  *   "wait_timeout_ms"  bound of every device-side wait (default 2000)
@@ -283,8 +289,9 @@ int swcs_energy_noalloc(swcs_ctx* ctx, const uint64_t* d_keys, const double* d_a
 /* Per-kernel device time with CUDA events recorded on the context's stream
  * around each launch (off by default).  Kinds: 0 gate/select kernel,
  * 1 energy, 2 hashed sigma scatter, 3 hashed pool gather, 4 table clear,
- * 5 other, 6 alpha-string row sweep, 7 grouping of the state by alpha string,
- * 8 adjoint gate.  swcs_profile_read synchronises, returns accumulated
+ * 5 other, 6 alpha-string row sweep or contraction of the density matrices,
+ * 7 grouping of the state by alpha string or sums over its pairs of
+ * determinants, 8 adjoint gate.  swcs_profile_read synchronises, returns accumulated
  * milliseconds and launch counts per kind (9 entries each; NULL to skip) and,
  * when reset != 0,
  * clears them together with the swcs_stats counters. */

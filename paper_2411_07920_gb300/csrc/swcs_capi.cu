@@ -84,8 +84,10 @@ struct swcs_ctx {
   int opt_screen_scatter = 1;  // a subset sweep marks and scatters only what the selected operators read
   bool screen_now = false;     // set around a subset sweep whose lists are built
 
-  // pairs of determinants (swcs_pairs.cu): string tables, grouped records, items
-  DevBuf pr_tab, pr_slot, pr_pos, pr_rec, pr_oth, pr_idx, pr_items;
+  // pairs of determinants (swcs_pairs.cu): string tables, grouped records, items; density matrices and the
+  // contraction's integrals and work arrays (swcs_rdm.cu)
+  DevBuf pr_tab, pr_slot, pr_pos, pr_rec, pr_oth, pr_idx, pr_items, rdm_tab, rdm_work, rdm_gamma;
+  int opt_pairs = -1;  // pool sweep from density matrices: -1 automatic, 0 never, 1 wherever it applies
 
   // external sigma table
   DevBuf ext;
@@ -732,8 +734,62 @@ int energy_rows(swcs_ctx* c, double* sig_out) {
   return sweep_rows(c, nullptr, -1, true, nullptr, true, sig_out);
 }
 
+// Whether the pool sweep of nd determinants goes through the density matrices.  Both paths' times in us, fitted to
+// the two sides measured at 12/4 with 24 determinants (61 by rows, 104 by matrices), 28/8 with 38,701 (1,950 and
+// 1,980), 46/10 with 33,333 (8,210 and 1,990) and 52/12 with 50,000 (39,100 and 2,800) and 10^6 (348,000 and
+// 33,800); the line lies where they meet:
+//   rows      every connected pair twice (1.18e5 visits per us) and every alpha string of the sector (8 ns)
+//   matrices  passes over them (2.1 MB per us), the two-body product (m^6), 8 ns per determinant, the pairs of
+//             the state (4.8e4 per us), and the contraction: 25 ns per determinant of a sparse state, at most
+//             that of full matrices (m^7).  A determinant of such states has some 300 neighbours within three
+//             excitations; one that fills a share of the sector has that share of all of them (1.5 times, as
+//             states crowd around the reference).
+bool use_density_matrices(swcs_ctx* c, int64_t nd) {
+  if (c->opt_sweep != 0 || c->opt_count_probes || c->opt_pairs == 0) return false;
+  if (c->no < 2 || nd > kMaxPairDets || !c->rdm_tab.p) return false;
+  if (c->opt_pairs == 1) return true;
+  if (c->NB <= 0 || c->NB > (1 << 22)) return true;  // no row sweep there: the hashed table is slower than either
+  const double n = (double)nd, m = c->n / 2, no = c->no, nv = c->nv;
+  const double single = no * nv, dbl = binom(c->no, 2) * binom(c->nv, 2), triple = binom(c->no, 3) * binom(c->nv, 3);
+  const double conn = 2.0 * single + 2.0 * dbl + single * single;
+  const double three = conn + 2.0 * triple + 2.0 * dbl * single;
+  const double rows = 60.0 + 0.008 * c->NA + 2.0 * n * (conn + 1.0) / 1.18e5;
+  const double hits = 300.0 + 1.5 * n / c->fci_dim * three;
+  const double mats = 110.0 + (double)rdm_gamma_doubles(c->n / 2) * 8.0 / 2.1e6 + 740.0 * std::pow(m / 26.0, 6) +
+                      n * (0.008 + hits / 9.6e4) + std::min(1070.0 * std::pow(m / 14.0, 7), 0.025 * n);
+  return mats < rows;
+}
+
+// Pool gradient and energy from the density matrices (swcs_rdm.cu); 1 when their memory cannot be had.
+int sweep_density(swcs_ctx* c, double* d_g, int64_t nd) {
+  const int m = c->n / 2;
+  const size_t gd = rdm_gamma_doubles(m);
+  if (ensure(c, c->rdm_gamma, gd * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8)) return 1;
+  RdmArgs a{};
+  const int r = pair_args(c, nd, false, &a.P);
+  if (r) return r;
+  rdm_layout(a, (double*)c->rdm_work.p, (double*)c->rdm_gamma.p, m);
+  a.V = rdm_tables((double*)c->rdm_tab.p, m);
+  a.pool_ops = (const uint8_t*)c->pool_dev.p;
+  a.pool_size = c->pool_size;
+  a.g = d_g;
+  CK(cudaMemsetAsync(c->rdm_gamma.p, 0, gd * 8, c->st));
+  CK(launch_k(c, kKGroup, [&] { return launch_pairs_gamma(a.P, nd, c->nsm, c->st); }));
+  CK(launch_k(c, kKRow, [&] { return launch_rdm_gradient(a, c->nsm, c->st); }));
+  c->launches += 4 + (c->no >= 3 ? 8 : 7);
+  CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(ctrl(c)->acc, ctrl(c)->eout, c->st); }));
+  c->stats[2] = c->stats[3] = c->stats[4] = 0;
+  return SWCS_OK;
+}
+
 int sweep(swcs_ctx* c, double* d_g, const uint32_t* sel = nullptr) {
   if (c->opt_sweep != 1) {
+    const int64_t nd = host_state_size(c);
+    if (nd < 0) return fail(c, SWCS_ERR_CUDA, "cannot read state size");
+    if (use_density_matrices(c, nd)) {
+      const int r = sweep_density(c, d_g, nd);
+      if (r != 1) return r;
+    }
     const int r = sweep_rows(c, d_g, -1, true, sel);
     if (r != 1) return r;
     if (c->opt_sweep == 2) return fail(c, SWCS_ERR_INVALID_ARG, "row sweep not applicable to this sector");
@@ -875,7 +931,8 @@ int swcs_destroy(swcs_ctx* c) {
                     &c->ck_keys, &c->ck_amps, &c->ck_n, &c->sn_keys, &c->sn_amps, &c->sn_n, &c->sigma, &c->nu0,
                     &c->nu1, &c->atab0, &c->atab1, &c->dth, &c->pool_dev, &c->selbits, &c->feat,
                     &c->ypred, &c->topk_hist, &c->topk_ctl, &c->occ, &c->prb, &c->ab_cnt, &c->ab_list,
-                    &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items};
+                    &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items,
+                    &c->rdm_tab, &c->rdm_work, &c->rdm_gamma};
   for (DevBuf* b : bufs) release(*b);
   if (c->pin) cudaFreeHost(c->pin);
   for (auto& e : c->ev_pending) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
@@ -911,6 +968,14 @@ int swcs_load_hamiltonian(swcs_ctx* c, const double* h_h, const double* h_g, int
   CK(cudaMemcpyAsync(c->h.p, h_h, n2 * 8, cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(c->gstage.p, h_g, n4 * 8, cudaMemcpyHostToDevice, c->st));
   CK(launch_k(c, kKOther, [&] { return launch_pack_hamiltonian((const double*)c->gstage.p, n, (double*)c->J.p, (double*)c->Ws.p, (double*)c->G.p, c->st); }));
+  if (c->no >= 2) {  // the density-matrix contraction's layout of the same integrals
+    if ((r = ensure(c, c->rdm_tab, rdm_table_doubles(n / 2) * 8))) return r;
+    CK(launch_k(c, kKOther, [&] {
+      return launch_rdm_tables((const double*)c->gstage.p, n, rdm_tables((double*)c->rdm_tab.p, n / 2), c->st);
+    }));
+  } else {
+    release(c->rdm_tab);
+  }
   std::vector<int> opd, ops1;
   build_pool(c, opd, ops1);
   {
@@ -1234,7 +1299,9 @@ int swcs_pool_gradients_dev(swcs_ctx* c, double* d_g_out, const int64_t* d_subse
     CK(launch_k(c, kKOther, [&] { return launch_subset_bits(d_subset, n_subset, (uint32_t*)c->selbits.p, c->pool_size, c->st); }));
     sel = (const uint32_t*)c->selbits.p;
     const int m = c->n / 2;
-    if (c->opt_screen_scatter && c->kab.p && m <= 32) {  // selected alpha-beta doubles per alpha pair
+    const int64_t nd = host_state_size(c);
+    if (nd < 0) return fail(c, SWCS_ERR_CUDA, "cannot read state size");
+    if (c->opt_screen_scatter && c->kab.p && m <= 32 && !use_density_matrices(c, nd)) {  // selected alpha-beta doubles per alpha pair
       const size_t m2 = (size_t)m * m;
       if ((r = ensure(c, c->ab_cnt, m2 * 4)) || (r = ensure(c, c->ab_list, m2 * m2 * 8))) return r;
       CK(launch_k(c, kKOther, [&] {
@@ -1563,6 +1630,9 @@ int swcs_set_option(swcs_ctx* c, const char* name, int64_t value) {
     if (value != 128 && value != 256 && value != 512 && value != 1024)
       return fail(c, SWCS_ERR_INVALID_ARG, "threads must be 128, 256, 512 or 1024");
     c->opt_threads = (int)value;
+  } else if (k == "pairs") {
+    if (value < -1 || value > 1) return fail(c, SWCS_ERR_INVALID_ARG, "pairs must be -1, 0 or 1");
+    c->opt_pairs = (int)value;
   } else if (k == "rows_l2") {
     c->opt_rows_l2 = value != 0;
   } else if (k == "cluster") {

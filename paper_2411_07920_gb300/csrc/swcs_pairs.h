@@ -1,4 +1,5 @@
-// Interface of the pair enumeration (swcs_pairs.cu).
+// Interface of the pair enumeration (swcs_pairs.cu) and of the density-matrix
+// pool gradient built on it (swcs_rdm.cu).
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -55,5 +56,37 @@ struct PairArgs {
 
 cudaError_t launch_pairs_energy(const PairArgs& a, int64_t n, int nsm, cudaStream_t st);
 cudaError_t launch_pairs_gamma(const PairArgs& a, int64_t n, int nsm, cudaStream_t st);
+
+// Tables of the Hamiltonian for the contraction, laid out once when it is loaded (m spatial orbitals, P = m(m-1)/2):
+//   vss [2][m][P][m]     g(p s, x s; y s, z s), pair (y < z), at ((s m + x) P + pair) m + p
+//   vos [2][m][m][m][m]  g(p s, x o; y o, z s), o = 1 - s, at (((s m + x) m + y) m + z) m + p
+//   v2s [2][P][P]        g(p s, q s; y s, z s)
+//   v2m [m^2][m^2]       g(p alpha, q beta; y alpha, z beta)
+// with g(p, x; y, z) = <px||yz>.
+struct RdmTables {
+  double *vss, *vos, *v2s, *v2m;
+};
+size_t rdm_table_doubles(int m);
+RdmTables rdm_tables(double* base, int m);
+cudaError_t launch_rdm_tables(const double* g_full, int n, const RdmTables& t, cudaStream_t st);
+
+struct RdmArgs {
+  PairArgs P;            // the density matrices and the state's counters
+  RdmTables V;
+  const uint8_t* pool_ops;
+  int64_t pool_size;
+  double* s_ss;          // [2][P][m][m]    contraction, operator order (rs, q, p)
+  double* s_ab;          // [m^2][m][m]     p alpha, q beta
+  double* s_ba;          // [m^2][m][m]     p beta, q alpha
+  double *g_ss, *g_ab;   // two-body density matrices [2][P][P], [m^2][m^2]
+  double *w_ss, *w_ab;   // their contractions with the integrals
+  double* gam;           // [2][m][m] one-body density matrix
+  double* lam;           // [2][m][m] <a+_r K_p>
+  double* g;             // the pool gradient
+};
+size_t rdm_work_doubles(int m);      // s_ss .. lam in one buffer
+size_t rdm_gamma_doubles(int m);     // the four density matrices
+void rdm_layout(RdmArgs& a, double* work, double* gamma, int m);
+cudaError_t launch_rdm_gradient(const RdmArgs& a, int nsm, cudaStream_t st);
 
 }  // namespace swcs

@@ -1,0 +1,631 @@
+// Pool gradient from the state's density matrices.
+//
+// For a real state and A_k = tau_k - tau_k^dag, g_k = 2 <psi|H A_k|psi>/<psi|psi>
+// = 2 <[H, tau_k]>/<psi|psi>: the commutator removes the part of H tau_k that is
+// disconnected, so only the one-, two- and three-body density matrices of the
+// state enter and no determinant outside the state is ever formed (the
+// three-body matrices come from swcs_pairs.cu).  With K_p = [a_p, H]
+//   = sum_k h_pk a_k + sum_{x, y<z} <px||yz> a+_x a_z a_y,
+//   <[H, a+_r a+_s a_q a_p]> = h-part(r;s;pq) - h-part(s;r;pq) + w(rs;pq) - S(r;s;pq) + S(s;r;pq)
+//                            + h-part(q;p;rs) - h-part(p;q;rs) - w(pq;rs) - S(q;p;rs) + S(p;q;rs),
+//   S(p;q;rs) = sum_{x, y<z} <px||yz> <a+_r a+_s a+_x a_q a_z a_y>,
+//   w(pq;rs)  = sum_{y<z} <pq||yz> <a+_r a+_s a_z a_y>,  h-part(p;q;rs) = sum_k h_pk <a+_r a+_s a_q a_k>,
+//   <[H, a+_r a_p]> = lam(r;p) - lam(p;r),  lam(p;r) = <a+_r K_p> = sum_k h_pk <a+_r a_k> + sum_x w(px;rx).
+//
+// S is the whole cost: sums over m^7-like index sets, but linear in the nonzero
+// elements of the three-body matrices (a few percent to a quarter of them are
+// nonzero for the truncated states of 46 and 52 spin-orbitals).  One CTA takes
+// one row T of a matrix, compacts its nonzeros into shared memory and hands
+// the list to its warps, one role of the row each; lanes are p, so a role's
+// use of an element reads the integrals over p (contiguous) and adds their
+// product with the element to R[q][p] in shared memory with one FP64 FMA
+// instruction.  A mixed row (t0 t1 of spin s, u of the other spin) has the roles
+//   rs = t0 t1, x = u        p, q of spin s
+//   rs = t1 u,  x = t0 ; rs = t0 u,  x = t1   with p, q of opposite spins, both ways
+// and a same-spin row the three choices of x; every role uses an element twice
+// (three times).  No two warps share an accumulator.  Bound by the FP64 pipe (a
+// warp's FMA takes 16 cycles of an SM's pipe; m <= 16 puts the two uses side by
+// side in one).  Whole pool sweep: 33.8 ms at 52/12 with 10^6 determinants (348 ms
+// by alpha-string rows), 2.8 ms there with 50,000 (39 ms), 2.0 ms at 46/10 with
+// 33,333 (8.2 ms); the contraction alone 20.9 + 2.5, 1.0 + 0.2 and 1.0 + 0.15 ms.
+// Accumulators in registers with q unrolled were 10 % faster on the densest of
+// these and 2.5 times slower on the others (bit tests of q dominated).
+#include <algorithm>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "swcs_device.cuh"
+#include "swcs_kernels.h"
+#include "swcs_pairs.h"
+
+namespace swcs {
+
+namespace {
+
+constexpr int kConThreads = 128;   // a warp per role of a mixed row
+constexpr int kSameThreads = 96;   // a warp per choice of x
+constexpr int kListCap = 1536;     // nonzeros of a row worked on at a time
+
+__host__ __device__ __forceinline__ size_t pairs_of(int m) { return (size_t)m * (m - 1) / 2; }
+__host__ __device__ __forceinline__ size_t triples_of(int m) { return (size_t)m * (m - 1) * (m - 2) / 6; }
+// rows padded to whole 32-byte sectors
+__host__ __device__ __forceinline__ size_t ld_of(size_t n) { return (n + 3) & ~(size_t)3; }
+
+__device__ __forceinline__ int pidx(int a, int b) { return a < b ? b * (b - 1) / 2 + a : a * (a - 1) / 2 + b; }
+
+__device__ __forceinline__ void pair_decode(int t, int& a, int& b) {  // t = b (b - 1) / 2 + a, a < b
+  b = (int)((1.0f + sqrtf(8.0f * (float)t + 1.0f)) * 0.5f);
+  while (b * (b - 1) / 2 > t) --b;
+  while ((b + 1) * b / 2 <= t) ++b;
+  a = t - b * (b - 1) / 2;
+}
+
+// ---------------------------------------------------------------- integrals
+__global__ void rdm_tables_kernel(const double* __restrict__ g, int n, RdmTables V) {
+  const int m = n / 2;
+  const long long P = (long long)pairs_of(m), m2 = (long long)m * m;
+  const long long n_ss = 2 * m2 * P, n_os = 2 * m2 * m2, n_2s = 2 * P * P, n_2m = m2 * m2;
+  auto at = [&](int p, int x, int y, int z) { return g[(((size_t)p * n + x) * n + y) * n + z]; };
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n_ss + n_os + n_2s + n_2m;
+       t += (long long)gridDim.x * blockDim.x) {
+    long long u = t;
+    int y, z;
+    if (u < n_ss) {
+      const int p = (int)(u % m), s = (int)(u / (m2 * P)), x = (int)((u / (m * P)) % m);
+      pair_decode((int)((u / m) % P), y, z);
+      V.vss[u] = at(2 * p + s, 2 * x + s, 2 * y + s, 2 * z + s);
+    } else if ((u -= n_ss) < n_os) {
+      const int p = (int)(u % m), s = (int)(u / (m2 * m2)), o = 1 - s;
+      z = (int)((u / m) % m);
+      y = (int)((u / m2) % m);
+      const int x = (int)((u / (m2 * m)) % m);
+      V.vos[u] = at(2 * p + s, 2 * x + o, 2 * y + o, 2 * z + s);
+    } else if ((u -= n_os) < n_2s) {
+      const int s = (int)(u / (P * P));
+      int p, q;
+      pair_decode((int)((u / P) % P), p, q);
+      pair_decode((int)(u % P), y, z);
+      V.v2s[u] = at(2 * p + s, 2 * q + s, 2 * y + s, 2 * z + s);
+    } else {
+      u -= n_2s;
+      const int pq = (int)(u / m2), yz = (int)(u % m2);
+      V.v2m[u] = at(2 * (pq / m), 2 * (pq % m) + 1, 2 * (yz / m), 2 * (yz % m) + 1);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- the lower triangles
+// Copies the upper triangles to the lower ones, 32 x 32 tiles (I <= J) of the matrix blockIdx.z (mixed, then
+// same-spin ones); a tile of zeros needs no copy, the matrices start as zeros.
+__global__ void __launch_bounds__(256) mirror_kernel(PairArgs A, int dim_mix, int dim_same) {
+  __shared__ double t[32][33];
+  const int I = blockIdx.y, J = blockIdx.x, z = blockIdx.z;
+  const int dim = z < 2 ? dim_mix : dim_same;
+  if (I > J || J * 32 >= dim) return;
+  double* M = z < 2 ? A.mix[z] : A.same[z - 2];
+  const size_t ld = z < 2 ? A.ld_mix : A.ld_same;
+  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+  bool any = false;
+#pragma unroll
+  for (int r = r0; r < 32; r += 8) {
+    const int i = I * 32 + r, j = J * 32 + c;
+    const double v = (i < dim && j < dim) ? M[(size_t)i * ld + j] : 0.0;
+    t[r][c] = v;
+    any |= v != 0.0;
+  }
+  if (!__syncthreads_or(any)) return;
+  for (int r = r0; r < 32; r += 8) {
+    const int j = J * 32 + r, i = I * 32 + c;  // element (j, i) = (i, j)
+    if (i < dim && j < dim && j > i) M[(size_t)j * ld + i] = t[c][r];
+  }
+}
+
+// ---------------------------------------------------------------- contraction
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }  // integer pipe
+
+// A row's nonzeros in shared memory: values, and their places as up to three orbitals in bytes.
+struct RowList {
+  double* val;
+  uint32_t* code;
+  int* cnt;
+};
+
+// Appends the nonzeros among elements [i0, i0 + batch) of a row (n elements) to the list, whole CTA.
+template <int kThreads, class F>
+__device__ __forceinline__ void scan_row(const double* row, int n, int i0, const RowList& L, F&& code_of) {
+  const int lane = threadIdx.x & 31;
+  double v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = i0 + k * kThreads + (int)threadIdx.x;
+    v[k] = i < n ? __ldcs(row + i) : 0.0;
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const bool nz = nonzero(v[k]);
+    const unsigned bal = __ballot_sync(0xffffffffu, nz);
+    if (!bal) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(L.cnt, __popc(bal));
+    base = __shfl_sync(0xffffffffu, base, 0) + __popc(bal & ((1u << lane) - 1u));
+    if (nz) {
+      L.val[base] = v[k];
+      L.code[base] = code_of(i0 + k * kThreads + (int)threadIdx.x);
+    }
+  }
+}
+
+// Shared memory of the contraction: accumulators [roles][m][m], the list, the pair decoding.
+__host__ __device__ constexpr size_t contract_smem(int m, int roles) {
+  return (size_t)roles * m * m * 8 + (size_t)kListCap * 12 + (size_t)m * (m - 1) / 2 * 2 + 16;
+}
+
+template <int kThreads>
+__device__ __forceinline__ void contract_init(double* acc, int n_acc, uint16_t* pr, int P) {
+  for (int t = threadIdx.x; t < n_acc; t += kThreads) acc[t] = 0.0;
+  for (int t = threadIdx.x; t < P; t += kThreads) {
+    int a, b;
+    pair_decode(t, a, b);
+    pr[t] = (uint16_t)(a | (b << 8));
+  }
+}
+
+// Adds an accumulator into the contraction and clears it.
+template <int kThreads>
+__device__ __forceinline__ void flush_acc(double* acc, int n, double* out, int neg) {
+  for (int t = threadIdx.x; t < n; t += kThreads) {
+    const double v = acc[t];
+    if (nonzero(v)) {
+      atomicAdd(&out[t], apply_sign(v, neg));
+      acc[t] = 0.0;
+    }
+  }
+}
+
+template <bool HALF>  // m <= 16: the two uses of an element in the two halves of a warp
+__global__ void __launch_bounds__(kConThreads) contract_mixed_kernel(RdmArgs A) {
+  extern __shared__ __align__(16) double sh[];
+  __shared__ unsigned s_row;
+  __shared__ int s_skip, s_cnt;
+  const int m = A.P.m, P = (int)pairs_of(m), dim = P * m, m2 = m * m;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int p = HALF ? lane & 15 : lane, half = HALF ? lane >> 4 : 0;
+  double* acc = sh;  // [5][q][p]: rs = t0 t1; x = t0, x = t1 (p of the other spin); x = t0, x = t1 (q of the other spin)
+  const RowList L{acc + 5 * m2, (uint32_t*)(acc + 5 * m2 + kListCap), &s_cnt};
+  uint16_t* pr = (uint16_t*)(L.code + kListCap);
+  contract_init<kConThreads>(acc, 5 * m2, pr, P);
+  const float inv = 1.0f / (float)P;
+  const size_t m3 = (size_t)m * m * m;
+  for (;;) {
+    __syncthreads();  // everyone is done with the last row
+    if (threadIdx.x == 0) {
+      const unsigned w = atomicAdd(&A.P.ctl->next_row, 1u);
+      s_row = w;
+      // the matrices are positive: no diagonal element, no row
+      s_skip = w < 2u * dim && !nonzero(A.P.mix[w & 1u][(size_t)(w >> 1) * (A.P.ld_mix + 1)]);
+      s_cnt = 0;
+    }
+    __syncthreads();
+    const unsigned w = s_row;
+    if (w >= 2u * dim) break;
+    if (s_skip) continue;
+    const int s = (int)(w & 1u), o = 1 - s, T = (int)(w >> 1);  // the two matrices' rows alternate
+    const double* row = A.P.mix[s] + (size_t)T * A.P.ld_mix;
+    const int u = T / P, tt = T - u * P, t0 = pr[tt] & 255, t1 = pr[tt] >> 8;
+    // this warp's integrals: warps 0..2 by (y, z) of the lower determinant, warp 3 by its pair for both x
+    const double* v = warp == 0 ? A.V.vos + ((size_t)s * m + u) * m3
+                    : warp == 1 ? A.V.vos + ((size_t)o * m + t0) * m3
+                    : warp == 2 ? A.V.vos + ((size_t)o * m + t1) * m3
+                                : A.V.vss + ((size_t)s * m + t0) * P * m;
+    const size_t step = (size_t)(t1 - t0) * P * m;
+    double* R = acc + warp * m2;
+    auto work = [&] {
+      __syncthreads();
+      const int cnt = s_cnt;
+      if (p < m) {
+        if (warp < 3) {
+          // y of spin s, z of the other: integrals at [z][y][p] for x = u, at [y][z][p] for x of spin s
+          const int sy = warp == 0 ? m : m2, sz = warp == 0 ? m2 : m;
+#pragma unroll 2
+          for (int k = 0; k < cnt; ++k) {
+            const double g = L.val[k];
+            const uint32_t c = L.code[k];
+            const int a = c & 255, b = (c >> 8) & 255, z = c >> 16;
+            if (HALF) {  // q = b, y = a and q = a, y = b
+              const int q = half ? a : b, y = half ? b : a;
+              R[q * m + p] += __ldg(&v[y * sy + z * sz + p]) * apply_sign(g, half);
+            } else {
+              const double va = __ldg(&v[a * sy + z * sz + p]), vb = __ldg(&v[b * sy + z * sz + p]);
+              R[b * m + p] += va * g;
+              R[a * m + p] -= vb * g;
+            }
+          }
+        } else {
+          double* R2 = R + m2;
+#pragma unroll 2
+          for (int k = 0; k < cnt; ++k) {
+            const double g = L.val[k];
+            const uint32_t c = L.code[k];
+            const int a = c & 255, b = (c >> 8) & 255, z = c >> 16, at = (b * (b - 1) / 2 + a) * m + p;
+            if (HALF) {
+              double* r = half ? R2 : R;
+              r[z * m + p] += __ldg(&v[at + (half ? step : 0)]) * g;
+            } else {
+              const double va = __ldg(&v[at]), vb = __ldg(&v[at + step]);
+              R[z * m + p] += va * g;
+              R2[z * m + p] += vb * g;
+            }
+          }
+        }
+      }
+      __syncthreads();
+    };
+    for (int i0 = 0; i0 < dim; i0 += 4 * kConThreads) {
+      scan_row<kConThreads>(row, dim, i0, L, [&](int i) {
+        const int z = (int)(((float)i + 0.5f) * inv);
+        return (uint32_t)pr[i - z * P] | ((uint32_t)z << 16);
+      });
+      __syncthreads();
+      if (s_cnt > kListCap - 4 * kConThreads) {
+        work();
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+      }
+    }
+    work();
+    // blocks of (q, p): rs = (alpha, beta) whatever the spin of the pair
+    const size_t rs0 = (size_t)(s == 0 ? t1 * m + u : u * m + t1) * m2;  // x = t0
+    const size_t rs1 = (size_t)(s == 0 ? t0 * m + u : u * m + t0) * m2;  // x = t1
+    double* ob = s == 0 ? A.s_ba : A.s_ab;  // p of the other spin, q of spin s
+    double* oa = s == 0 ? A.s_ab : A.s_ba;  // p of spin s, q of the other
+    flush_acc<kConThreads>(acc, m2, A.s_ss + ((size_t)s * P + tt) * m2, 0);
+    flush_acc<kConThreads>(acc + m2, m2, ob + rs0, s == 0);
+    flush_acc<kConThreads>(acc + 2 * m2, m2, ob + rs1, s == 1);
+    flush_acc<kConThreads>(acc + 3 * m2, m2, oa + rs0, s == 1);
+    flush_acc<kConThreads>(acc + 4 * m2, m2, oa + rs1, s == 0);
+  }
+}
+
+__global__ void __launch_bounds__(kSameThreads) contract_same_kernel(RdmArgs A) {
+  extern __shared__ __align__(16) double sh[];
+  __shared__ int s_cnt;
+  const int m = A.P.m, P = (int)pairs_of(m), dim = (int)triples_of(m), m2 = m * m;
+  const int warp = threadIdx.x >> 5, p = threadIdx.x & 31;
+  double* acc = sh;  // [3][q][p], by x
+  const RowList L{acc + 3 * m2, (uint32_t*)(acc + 3 * m2 + kListCap), &s_cnt};
+  uint16_t* pr = (uint16_t*)(L.code + kListCap);
+  contract_init<kSameThreads>(acc, 3 * m2, pr, P);
+  for (int w = blockIdx.x; w < 2 * dim; w += gridDim.x) {
+    const int s = w & 1, T = w >> 1;
+    const double* row = A.P.same[s] + (size_t)T * A.P.ld_same;
+    if (!nonzero(row[T])) continue;
+    __syncthreads();  // tables built; everyone is done with the last row
+    if (threadIdx.x == 0) s_cnt = 0;
+    int t2 = 2;
+    while ((t2 + 1) * t2 * (t2 - 1) / 6 <= T) ++t2;
+    const uint32_t t01 = pr[T - t2 * (t2 - 1) * (t2 - 2) / 6];
+    const int t0 = t01 & 255, t1 = t01 >> 8;
+    const double* v = A.V.vss + ((size_t)s * m + (warp == 0 ? t0 : warp == 1 ? t1 : t2)) * P * m;
+    double* R = acc + warp * m2;
+    __syncthreads();
+    auto work = [&] {
+      __syncthreads();
+      const int cnt = s_cnt;
+      if (p < m) {
+#pragma unroll 2
+        for (int k = 0; k < cnt; ++k) {
+          const double g = L.val[k];
+          const uint32_t c = L.code[k];
+          const int x = c & 255, y = (c >> 8) & 255, z = c >> 16;
+          const double vx = __ldg(&v[(z * (z - 1) / 2 + y) * m + p]), vy = __ldg(&v[(z * (z - 1) / 2 + x) * m + p]);
+          const double vz = __ldg(&v[(y * (y - 1) / 2 + x) * m + p]);
+          R[x * m + p] += vx * g;
+          R[y * m + p] -= vy * g;
+          R[z * m + p] += vz * g;
+        }
+      }
+      __syncthreads();
+    };
+    for (int i0 = 0; i0 < dim; i0 += 4 * kSameThreads) {
+      scan_row<kSameThreads>(row, dim, i0, L, [&](int i) {
+        int z = (int)cbrtf(6.0f * (float)i + 1.0f) + 1;  // z (z - 1) (z - 2) / 6 <= i
+        while (z * (z - 1) * (z - 2) / 6 > i) --z;
+        while ((z + 1) * z * (z - 1) / 6 <= i) ++z;
+        return (uint32_t)pr[i - z * (z - 1) * (z - 2) / 6] | ((uint32_t)z << 16);
+      });
+      __syncthreads();
+      if (s_cnt > kListCap - 4 * kSameThreads) {
+        work();
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+      }
+    }
+    work();
+    double* base = A.s_ss + (size_t)s * P * m2;
+    flush_acc<kSameThreads>(acc, m2, base + (size_t)pidx(t1, t2) * m2, 0);
+    flush_acc<kSameThreads>(acc + m2, m2, base + (size_t)pidx(t0, t2) * m2, 1);
+    flush_acc<kSameThreads>(acc + 2 * m2, m2, base + (size_t)pidx(t0, t1) * m2, 0);
+  }
+}
+
+// ---------------------------------------------------------------- two-body density matrices by partial traces
+// The number of electrons of each spin is fixed: the trace of the mixed block over its single is no times the
+// same-spin pair matrix, its trace over one orbital of the pair (no - 1) times the opposite-spin one.
+__global__ void trace_kernel(RdmArgs A) {
+  const int m = A.P.m, no = A.P.H.no;
+  const long long P = (long long)pairs_of(m), m2 = (long long)m * m;
+  const size_t ld = A.P.ld_mix;
+  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * P * P + m2 * m2;
+       t += (long long)gridDim.x * blockDim.x) {
+    double v = 0.0;
+    if (t < 2 * P * P) {
+      const int s = (int)(t / (P * P));
+      const double* M = A.P.mix[s] + (size_t)((t / P) % P) * ld + (size_t)(t % P);
+      for (int u = 0; u < m; ++u) v += M[(size_t)u * P * (ld + 1)];
+      A.g_ss[t] = v / no;
+    } else {
+      const long long u = t - 2 * P * P;
+      const int a = (int)(u / (m2 * m)), c = (int)((u / m2) % m), a2 = (int)((u / m) % m), c2 = (int)(u % m);
+      for (int x = 0; x < m; ++x) {
+        if (x == a || x == a2) continue;
+        const double w = A.P.mix[0][(size_t)(c * P + pidx(a, x)) * ld + c2 * P + pidx(a2, x)];
+        v += ((x > a) == (x > a2)) ? w : -w;
+      }
+      A.g_ab[u] = v / (no - 1);
+    }
+  }
+}
+
+// C[i][j] += sum_k A[i][k] B[j][k], n x n, 32 x 32 tiles; blockIdx.z picks the block (two same-spin, one mixed) and
+// one of kTwoSplit ranges of k (more CTAs than a tile count alone gives: 484 at 52 spin-orbitals); C starts as zeros.
+constexpr int kTwoSplit = 3;
+__global__ void __launch_bounds__(256) two_body_kernel(RdmArgs A) {
+  __shared__ double sa[32][33], sb[32][33];
+  const int m = A.P.m, P = (int)pairs_of(m);
+  const int which = blockIdx.z / kTwoSplit, part = blockIdx.z % kTwoSplit;
+  const int n = which < 2 ? P : m * m;
+  const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
+  if (i0 >= n || j0 >= n) return;
+  const int kper = ((n + 31) / 32 + kTwoSplit - 1) / kTwoSplit * 32, kb = part * kper, ke = min(n, kb + kper);
+  const size_t b = (size_t)which * P * P;
+  const double* X = which < 2 ? A.V.v2s + b : A.V.v2m;
+  const double* Y = which < 2 ? A.g_ss + b : A.g_ab;
+  double* C = which < 2 ? A.w_ss + b : A.w_ab;
+  const int c = threadIdx.x & 31, r = threadIdx.x >> 5;  // 8 rows of 32; a thread has rows r, r + 8, r + 16, r + 24
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int k0 = kb; k0 < ke; k0 += 32) {
+    for (int q = r; q < 32; q += 8) {
+      const bool kin = k0 + c < n;
+      sa[q][c] = (kin && i0 + q < n) ? X[(size_t)(i0 + q) * n + k0 + c] : 0.0;
+      sb[q][c] = (kin && j0 + q < n) ? Y[(size_t)(j0 + q) * n + k0 + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < 32; ++k) {
+      const double y = sb[c][k];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] += sa[r + 8 * q][k] * y;
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (kb < ke && i0 + r + 8 * q < n && j0 + c < n) atomicAdd(&C[(size_t)(i0 + r + 8 * q) * n + j0 + c], acc[q]);
+}
+
+// Blocks as spin-orbital quantities (p = 2 spatial + spin).
+struct Views {
+  const RdmArgs& A;
+  int m, P;
+  __device__ double g2(int r, int s, int p, int q) const {  // <a+_r a+_s a_q a_p>, r != s, p != q
+    double sg = 1.0;
+    if ((r & 1) == (s & 1)) {
+      if (r > s) sg = -sg;
+      if (p > q) sg = -sg;
+      return sg * __ldg(&A.g_ss[(size_t)(r & 1) * P * P + (size_t)pidx(r >> 1, s >> 1) * P + pidx(p >> 1, q >> 1)]);
+    }
+    if (r & 1) { const int t = r; r = s; s = t; sg = -sg; }
+    if (p & 1) { const int t = p; p = q; q = t; sg = -sg; }
+    return sg * __ldg(&A.g_ab[(size_t)((r >> 1) * m + (s >> 1)) * m * m + (p >> 1) * m + (q >> 1)]);
+  }
+  __device__ double w(int p, int q, int r, int s) const {  // w(pq; rs)
+    double sg = 1.0;
+    if (p == q || r == s) return 0.0;
+    if ((r & 1) == (s & 1)) {
+      if (p > q) sg = -sg;
+      if (r > s) sg = -sg;
+      return sg * A.w_ss[(size_t)(r & 1) * P * P + (size_t)pidx(p >> 1, q >> 1) * P + pidx(r >> 1, s >> 1)];
+    }
+    if (p & 1) { const int t = p; p = q; q = t; sg = -sg; }
+    if (r & 1) { const int t = r; r = s; s = t; sg = -sg; }
+    return sg * A.w_ab[(size_t)((p >> 1) * m + (q >> 1)) * m * m + (r >> 1) * m + (s >> 1)];
+  }
+  __device__ double S(int p, int q, int r, int s) const {  // S(p; q; rs)
+    const int at = (q >> 1) * m + (p >> 1);
+    if ((r & 1) == (s & 1)) {
+      const double v = A.s_ss[((size_t)(r & 1) * P + pidx(r >> 1, s >> 1)) * m * m + at];
+      return r < s ? v : -v;
+    }
+    double sg = 1.0;
+    if (r & 1) { const int t = r; r = s; s = t; sg = -1.0; }
+    return sg * ((p & 1) ? A.s_ba : A.s_ab)[(size_t)((r >> 1) * m + (s >> 1)) * m * m + at];
+  }
+};
+
+// The contraction starts from minus the one-body part: S(p; q; rs) -= sum_k h_pk <a+_r a+_s a_q a_k> over the
+// orbitals k of p's spin.  One CTA per (block, rs), threads over (q, p).
+__global__ void __launch_bounds__(256) one_body_part_kernel(RdmArgs A) {
+  __shared__ double hs[kMaxSpin * kMaxSpin];
+  __shared__ double gk[kMaxSpin * kMaxSpin];
+  const int m = A.P.m, P = (int)pairs_of(m), n = 2 * m;
+  const Views v{A, m, P};
+  int b = blockIdx.x, r, s, sp, sq;  // rs and the spins of p and q
+  double* out;
+  if (b < 2 * P) {
+    sp = sq = b >= P;
+    pair_decode(b % P, r, s);
+    r = 2 * r + sp;
+    s = 2 * s + sp;
+    out = A.s_ss + (size_t)b * m * m;
+  } else {
+    b -= 2 * P;
+    sp = b >= m * m;  // s_ab: p alpha; s_ba: p beta
+    sq = 1 - sp;
+    if (sp) b -= m * m;
+    r = 2 * (b / m);
+    s = 2 * (b % m) + 1;
+    out = (sp ? A.s_ba : A.s_ab) + (size_t)b * m * m;
+  }
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    const int i = t / m, k = t % m;
+    hs[t] = A.P.H.h[(2 * i + sp) * n + 2 * k + sp];
+    gk[t] = (sp == sq && i == k) ? 0.0 : v.g2(r, s, 2 * k + sp, 2 * i + sq);  // [q][k]
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    const int q = t / m, p = t % m;
+    double x = 0.0;
+    for (int k = 0; k < m; ++k) x += hs[k * m + p] * gk[q * m + k];  // h is symmetric
+    out[t] = -x;
+  }
+}
+
+// One-body density matrix: partial trace of the opposite-spin pair matrix.
+__global__ void one_rdm_kernel(RdmArgs A) {
+  const int m = A.P.m;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 2 * m * m; t += gridDim.x * blockDim.x) {
+    const int s = t / (m * m), a = (t / m) % m, c = t % m;
+    double g = 0.0;
+    for (int b = 0; b < m; ++b)
+      g += s == 0 ? A.g_ab[(size_t)(a * m + b) * m * m + c * m + b] : A.g_ab[(size_t)(b * m + a) * m * m + b * m + c];
+    A.gam[t] = g / A.P.H.no;
+  }
+}
+
+// lam(p; r) and the energy numerator, one warp per (p, r).
+__global__ void __launch_bounds__(256) lambda_kernel(RdmArgs A) {
+  const int m = A.P.m, P = (int)pairs_of(m), n = 2 * m, lane = threadIdx.x & 31;
+  const Views v{A, m, P};
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (t >= 2 * m * m) return;
+  const int s = t / (m * m), p = 2 * ((t / m) % m) + s, r = 2 * (t % m) + s;
+  double one = 0.0, two = 0.0;
+  if (lane < m) one = A.P.H.h[p * n + 2 * lane + s] * A.gam[(size_t)s * m * m + (r >> 1) * m + lane];
+  for (int x = lane; x < n; x += 32)
+    if (x != p && x != r) two += v.w(p, x, r, x);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    one += __shfl_xor_sync(0xffffffffu, one, o);
+    two += __shfl_xor_sync(0xffffffffu, two, o);
+  }
+  if (lane == 0) {
+    A.lam[t] = one + two;
+    if (p == r) atomicAdd(&A.P.acc[0], one + 0.5 * two);
+  }
+}
+
+__global__ void __launch_bounds__(256) assemble_kernel(RdmArgs A) {
+  const int m = A.P.m, P = (int)pairs_of(m);
+  const Views v{A, m, P};
+  const double f = 2.0 / A.P.acc[1];
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < A.pool_size; k += (int64_t)gridDim.x * blockDim.x) {
+    const uint8_t* op = A.pool_ops + 5 * k;
+    double t;
+    if (op[0] == 1) {
+      const int p = op[1], r = op[2], s = p & 1;
+      const double* l = A.lam + (size_t)s * m * m;
+      t = l[(r >> 1) * m + (p >> 1)] - l[(p >> 1) * m + (r >> 1)];
+    } else {
+      const int p = op[1], q = op[2], r = op[3], s = op[4];
+      t = (v.w(r, s, p, q) - v.w(p, q, r, s)) + (v.S(s, r, p, q) - v.S(r, s, p, q)) + (v.S(p, q, r, s) - v.S(q, p, r, s));
+    }
+    A.g[k] = f * t;
+  }
+}
+
+cudaError_t launch_contract(const RdmArgs& a, int nsm, cudaStream_t st) {
+  const int m = a.P.m;
+  const size_t s1 = contract_smem(m, 5), s2 = contract_smem(m, 3);
+  const auto mixed = m <= 16 ? contract_mixed_kernel<true> : contract_mixed_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s1);
+  if (e != cudaSuccess) return e;
+  mixed<<<(unsigned)std::min<size_t>(2 * pairs_of(m) * m, (size_t)8 * nsm), kConThreads, s1, st>>>(a);
+  if (a.P.H.no >= 3) {
+    e = cudaFuncSetAttribute(contract_same_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s2);
+    if (e != cudaSuccess) return e;
+    contract_same_kernel<<<(unsigned)std::min<size_t>(2 * triples_of(m), (size_t)8 * nsm), kSameThreads, s2, st>>>(a);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t rdm_table_doubles(int m) {
+  const size_t P = pairs_of(m), m2 = (size_t)m * m;
+  return 2 * m2 * P + 2 * m2 * m2 + 2 * P * P + m2 * m2;
+}
+
+RdmTables rdm_tables(double* base, int m) {
+  const size_t P = pairs_of(m), m2 = (size_t)m * m;
+  RdmTables t;
+  t.vss = base;
+  t.vos = t.vss + 2 * m2 * P;
+  t.v2s = t.vos + 2 * m2 * m2;
+  t.v2m = t.v2s + 2 * P * P;
+  return t;
+}
+
+cudaError_t launch_rdm_tables(const double* g_full, int n, const RdmTables& t, cudaStream_t st) {
+  rdm_tables_kernel<<<1216, 256, 0, st>>>(g_full, n, t);
+  return cudaGetLastError();
+}
+
+
+size_t rdm_work_doubles(int m) {
+  const size_t P = pairs_of(m), m2 = (size_t)m * m;
+  return 2 * P * m2 + 2 * m2 * m2 + 2 * (2 * P * P + m2 * m2) + 4 * m2;
+}
+
+size_t rdm_gamma_doubles(int m) {
+  const size_t d1 = pairs_of(m) * m, d2 = triples_of(m);
+  return 2 * (d1 * ld_of(d1) + d2 * ld_of(d2));
+}
+
+void rdm_layout(RdmArgs& a, double* work, double* gamma, int m) {
+  const size_t P = pairs_of(m), m2 = (size_t)m * m, d1 = P * m, d2 = triples_of(m);
+  a.s_ss = work;
+  a.s_ab = a.s_ss + 2 * P * m2;
+  a.s_ba = a.s_ab + m2 * m2;
+  a.g_ss = a.s_ba + m2 * m2;
+  a.g_ab = a.g_ss + 2 * P * P;
+  a.w_ss = a.g_ab + m2 * m2;
+  a.w_ab = a.w_ss + 2 * P * P;
+  a.gam = a.w_ab + m2 * m2;
+  a.lam = a.gam + 2 * m2;
+  a.P.ld_mix = ld_of(d1);
+  a.P.ld_same = ld_of(d2);
+  a.P.mix[0] = gamma;
+  a.P.mix[1] = a.P.mix[0] + d1 * a.P.ld_mix;
+  a.P.same[0] = a.P.mix[1] + d1 * a.P.ld_mix;
+  a.P.same[1] = a.P.same[0] + d2 * a.P.ld_same;
+}
+
+cudaError_t launch_rdm_gradient(const RdmArgs& a, int nsm, cudaStream_t st) {
+  const int m = a.P.m, P = (int)pairs_of(m);
+  const int d1 = P * m, d2 = a.P.H.no >= 3 ? (int)triples_of(m) : 0;
+  mirror_kernel<<<dim3((d1 + 31) / 32, (d1 + 31) / 32, d2 ? 4 : 2), 256, 0, st>>>(a.P, d1, d2);
+  trace_kernel<<<1216, 256, 0, st>>>(a);
+  one_body_part_kernel<<<2 * P + 2 * m * m, 256, 0, st>>>(a);
+  one_rdm_kernel<<<(2 * m * m + 127) / 128, 128, 0, st>>>(a);
+  cudaError_t e = launch_contract(a, nsm, st);
+  if (e != cudaSuccess) return e;
+  const int nt = (m * m + 31) / 32;
+  e = cudaMemsetAsync(a.w_ss, 0, (2 * pairs_of(m) * pairs_of(m) + (size_t)m * m * m * m) * 8, st);
+  if (e != cudaSuccess) return e;
+  two_body_kernel<<<dim3(nt, nt, 3 * kTwoSplit), 256, 0, st>>>(a);
+  lambda_kernel<<<(2 * m * m + 7) / 8, 256, 0, st>>>(a);
+  assemble_kernel<<<(unsigned)std::min<int64_t>((a.pool_size + 255) / 256, 1216), 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace swcs

@@ -1,5 +1,6 @@
-"""Energy and sigma_D-based gradients from the pairs of the state's determinants
-(option "energy" 0) against the oracle: orbital counts at the edges of the kernels' layouts (16
+"""Energy, sigma_D-based gradients and the pool sweep from the pairs of the
+state's determinants (options "energy" 0 and "pairs" 1) against the oracle and
+against the row sweep: orbital counts at the edges of the kernels' layouts (16
 and 17 spatial orbitals, 32), two electrons of a spin (no same-spin triples),
 more electrons than holes, one determinant, states whose groups cross the
 32-determinant items, and determinants without any order or connection."""
@@ -17,6 +18,13 @@ def _check(c, w, k, a, mode="both"):
     e0, n0 = O.energy(w.n_so, w.h, w.g, k, a)
     e, n2 = c.energy()
     assert abs(e - e0) < TOL and abs(n2 - n0) < TOL * max(1.0, n0)
+    c.set_option("pairs", 1)
+    g = c.pool_gradients()
+    es, n2s = c.sweep_energy()
+    c.set_option("pairs", -1)
+    go = O.pool_gradients(w.n_so, w.h, w.g, k, a)
+    assert np.abs(g - go).max() < TOL
+    assert abs(es - e0) < TOL and abs(n2s - n0) < TOL * max(1.0, n0)
 
 
 @pytest.mark.parametrize("n_so,n_e,n_ops,n_keep", [
@@ -63,8 +71,34 @@ def test_pairs_arbitrary_states(n_so, n_e, n):
         _check(c, w, k, a)
 
 
-def test_one_electron_of_each_spin():
-    """One electron of each spin."""
+def test_pairs_agree_with_rows_and_subset():
+    """A larger state: both sweeps, the subset form, and an untouched entry outside the subset."""
+    import torch
+
+    from paper_2411_07920_gb300 import swcs
+    w = I.small_case(40, 10, 80, 23, n_keep=20_000)
+    with swcs.Context() as c:
+        c.load_hamiltonian(w.h, w.g, w.n_so, w.n_e)
+        c.apply_ansatz(w.ops, w.theta, 20_000)
+        out = []
+        for pairs in (0, 1):
+            c.set_option("pairs", pairs)
+            out.append((c.pool_gradients(), c.sweep_energy()))
+        assert np.abs(out[0][0] - out[1][0]).max() < TOL
+        assert abs(out[0][1][0] - out[1][1][0]) < TOL
+        sub = torch.arange(3, c.pool_size(), 7, dtype=torch.int64, device="cuda")
+        g = torch.full((c.pool_size(),), 7.0, dtype=torch.float64, device="cuda")
+        c.pool_gradients_dev(g, sub)
+        g = g.cpu().numpy()
+        s = sub.cpu().numpy()
+        assert np.abs(g[s] - out[0][0][s]).max() < TOL
+        rest = np.ones(len(g), bool)
+        rest[s] = False
+        assert (g[rest] == 7.0).all()
+
+
+def test_pairs_do_not_apply():
+    """One electron of each spin: no three-body matrix; the option leaves the row sweep in place."""
     from paper_2411_07920_gb300 import swcs
     w = I.small_case(12, 2, 6, 3)
     with swcs.Context() as c:
