@@ -183,9 +183,12 @@ int swcs_sweep_energy(swcs_ctx* ctx, double* h_e_out, double* h_norm2_out);
  * magnitude criterion drops them): without a cut the projector is the
  * identity on the reachable determinants, so the derivative is exact, also
  * at theta_g = 0 where the gate's partner determinants have c = 0.
- * The forward pass keeps a copy of the state every ckpt_every gates
- * (ckpt_every <= 0: 20); the backward pass replays each segment from its
- * checkpoint.  Leaves the final state in the context. */
+ * The forward pass records every gate's rotated blocks and dropped
+ * determinants on a tape, which the backward pass reads in reverse.  Where a
+ * tape of all gates would take more than an eighth of the free device memory
+ * (option "adjoint_tape_mb"), the forward pass keeps a copy of the state every
+ * ckpt_every gates instead (ckpt_every <= 0: 20) and each segment is replayed
+ * with its tape.  Leaves the final state in the context. */
 int swcs_energy_grad(swcs_ctx* ctx, const uint8_t* h_ops, const double* h_theta, int n_ops, int64_t n_keep,
                      int ckpt_every, double* h_e_out, double* h_dtheta_out);
 
@@ -249,7 +252,10 @@ int swcs_probe_counts(swcs_ctx* ctx, int64_t* h_out4, int reset);
  *              before its first grid barrier so the others' bounded waits
  *              run out (-1, default: off); the call then returns
  *              SWCS_ERR_TIMEOUT and the context stays usable
- *   "gate_blocks"   CTAs of the persistent gate kernel (0, default: whole device)
+ *   "gate_blocks"   CTAs of the persistent gate kernel (0, default: by the
+ *              state's size, up to the whole device)
+ *   "adjoint_tape_mb"  bound of the adjoint's tape in MiB (0, default: an
+ *              eighth of the free device memory)
  *   "row_clusters"  clusters of the row sweep (0, default: as many as fit)
  *   "count_probes"  1: count hash probes (swcs_probe_counts); 0 (default)
  *   "screen_scatter" subset sweeps of swcs_pool_gradients_dev: 1 (default)

@@ -13,6 +13,7 @@
 #include "../../include/swcs.h"
 #include "swcs_device.cuh"
 #include "swcs_kernels.h"
+#include "swcs_gates.h"
 #include "swcs_pairs.h"
 
 using namespace swcs;
@@ -76,8 +77,13 @@ struct swcs_ctx {
   int opt_gate_threads = kAnsatzThreads;  // threads per gate-kernel CTA (batched instances: kAnsatzThreadsShared)
   int opt_row_clusters = 0;  // clusters of the row sweep (0: as many as fit)
 
-  // adjoint: checkpoints, per-gate snapshots of one segment, sigma, nu, indices, gradient
-  DevBuf ck_keys, ck_amps, ck_n, sn_keys, sn_amps, sn_n, sigma, nu0, nu1, atab0, atab1, dth;
+  // in-place gate sequence: second amplitude array, partners put aside, free positions, positions of the output
+  DevBuf amps_c, low_keys, low_amps, low_rec, ring, out_pos, band, band_slots;
+  int64_t max_state = 0;    // determinants the state buffers are sized for
+  int cluster_ok[17] = {};  // clusters of k gate CTAs: 0 unknown, 1 fit, -1 do not
+  // adjoint: checkpoints, tape of a segment, sigma, nu by position, nu and index of a checkpoint, gradient
+  DevBuf ck_keys, ck_amps, ck_n, tp_pos, tp_x, tp_drop, tp_start, sigma, nu0, nu1, atab0, dth;
+  int64_t opt_tape_mb = 0;  // bound of the tape's memory (0: an eighth of the device's free memory)
   DevBuf prb;  // swcs_sigma_at: requested alpha strings, ranges, beta ranks and outputs
   DevBuf ab_cnt, ab_list;  // screened sweep: selected alpha-beta doubles per alpha pair
   DevBuf selhist;          // gate kernel: radix-select histograms (two sets of 12 passes x 4096 bins)
@@ -121,6 +127,8 @@ struct Ctrl {
   int err;
   GridBar bar;
   unsigned long long ctr[12];
+  unsigned long long gate_ctr[3 * kGateCtrN + 1];  // in-place gate sequence
+  unsigned long long zeros;                        // exactly zero amplitudes kept by the adjoint's projectors
   long long stats[8];
   double acc[2];
   PairCtl pairs;  // right after acc: one memset clears both
@@ -351,8 +359,49 @@ int ensure_state_buffers(swcs_ctx* c, int64_t max_state) {
     if ((r = ensure(c, c->tab1, tcap * sizeof(IdxSlot)))) return r;
     c->cap = cap;
     c->tab_mask = tcap - 1;
+    c->max_state = std::max<int64_t>(max_state, 1);
   }
-  return ensure(c, c->selhist, kAnsatzHistWords * 4);  // the gate kernel's select histograms
+  return ensure(c, c->selhist, std::max(kAnsatzHistWords, kGateHistWords) * 4);  // the gate kernels' select histograms
+}
+
+// Entries kept per bin around the cut: a bin near it holds about one determinant in 10^5.
+int band_slots_for(int64_t max_state) { return max_state <= 16384 ? 8 : 32; }
+
+// Work arrays of the in-place gate sequence for the state buffers' size N.  Positions: N determinants kept, up to N
+// new ones of a pass, N dropped in the pass before and N in this one, which are free two passes later: 4 N.  Its index
+// (tab1 as 8-byte slots: at least 4 N) holds the determinants kept and dropped ones' slots until it is built anew.
+int ensure_gate_buffers(swcs_ctx* c) {
+  const size_t n = (size_t)c->max_state, np = 4 * n + 64;
+  int r;
+  if ((r = ensure(c, c->keys_b, np * 8)) || (r = ensure(c, c->amps_b, np * 8)) || (r = ensure(c, c->amps_c, np * 8)) ||
+      (r = ensure(c, c->low_keys, n * 8)) || (r = ensure(c, c->low_amps, n * 8)) || (r = ensure(c, c->low_rec, n * 4)) ||
+      (r = ensure(c, c->ring, pow2_at_least(np) * 4)) || (r = ensure(c, c->band, 3 * kBandWords * 4)) ||
+      (r = ensure(c, c->band_slots, (size_t)3 * kBandBins * band_slots_for(c->max_state) * sizeof(BandEntry))))
+    return r;
+  return SWCS_OK;
+}
+
+constexpr int64_t kMaxInPlace = (int64_t)1 << 28;  // positions (four times that) fit 31 bits
+
+// CTAs of a gate-sequence or backward launch: up to 16 form one cluster where the device takes such clusters
+// (barriers of a fraction of a microsecond), larger states and launches with test hooks use a cooperative grid.
+// Measured per gate: see swcs_gates.cu.
+void gate_launch_shape(swcs_ctx* c, int per_sm, int* nblocks, bool* clustered) {
+  const int64_t want = (c->max_state + 2047) / 2048;
+  *clustered = false;
+  if (c->opt_skip_arrive < 0 && c->opt_gate_blocks == 0 && want <= 8) {
+    const int k = (int)std::max<int64_t>(1, std::min<int64_t>((c->max_state + 1023) / 1024, 16));
+    if (c->cluster_ok[k] == 0) c->cluster_ok[k] = gate_cluster_fits(k) > 0 ? 1 : -1;
+    if (c->cluster_ok[k] > 0) {
+      *nblocks = k;
+      *clustered = true;
+      return;
+    }
+  }
+  int nb = c->nsm * std::max(per_sm, 1);
+  if (c->opt_gate_blocks > 0) nb = std::min(nb, c->opt_gate_blocks);
+  else nb = (int)std::max<int64_t>(std::min<int64_t>(nb, (c->max_state + 511) / 512), std::min(nb, 8));
+  *nblocks = nb;
 }
 
 int64_t max_state_for(swcs_ctx* c, int64_t n_keep, int n_ops, int64_t n_now) {
@@ -363,13 +412,19 @@ int64_t max_state_for(swcs_ctx* c, int64_t n_keep, int n_ops, int64_t n_now) {
   return (int64_t)bound;
 }
 
+// |c| >= eps <=> abs bit pattern >= eps's bit pattern (IEEE-754 order of non-negative doubles).
 // keep_zeros: determinants a gate reaches with an exactly zero amplitude stay
 // in the kept set (ranked below every nonzero |c|) unless a criterion cuts
 // them -- the projectors of the adjoint need them (a partner at theta = 0 has
 // c = 0 but a nonzero derivative); the magnitude criterion still drops them.
-// The gate kernel's arguments for this context (no launch).
-AnsatzArgs gate_args(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, int64_t n_keep, bool reset,
-                     uint64_t* snap_keys, double* snap_amps, long long* snap_n, int64_t snap_stride, bool keep_zeros) {
+uint64_t min_abs_bits(const swcs_ctx* c, bool keep_zeros) {
+  uint64_t eb = 0;
+  std::memcpy(&eb, &c->trunc_eps, 8);
+  return c->trunc_eps > 0.0 ? eb : (keep_zeros ? 0ull : 1ull);
+}
+
+// The rebuilding gate kernel's arguments for this context (no launch).
+AnsatzArgs gate_args(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, int64_t n_keep, bool reset) {
   AnsatzArgs a{};
   a.keys_a = (uint64_t*)c->keys_a.p;
   a.amps_a = (double*)c->amps_a.p;
@@ -384,11 +439,7 @@ AnsatzArgs gate_args(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int 
   a.cs = d_cs;
   a.n_ops = n_ops;
   a.n_keep = n_keep;
-  {  // |c| >= eps <=> abs bit pattern >= eps's bit pattern (IEEE-754 order of non-negative doubles)
-    uint64_t eb = 0;
-    std::memcpy(&eb, &c->trunc_eps, 8);
-    a.min_abs_bits = (c->trunc_eps > 0.0) ? eb : (keep_zeros ? 0ull : 1ull);
-  }
+  a.min_abs_bits = min_abs_bits(c, false);
   a.reset_to_hf = reset ? 1 : 0;
   a.hf = (c->ne >= 64) ? ~0ull : ((1ull << c->ne) - 1ull);
   Ctrl* k = ctrl(c);
@@ -401,25 +452,82 @@ AnsatzArgs gate_args(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int 
   a.timeout_ns = c->opt_timeout_ns;
   a.skip_arrive_block = c->opt_skip_arrive;
   a.probe_ctr = c->opt_count_probes ? &k->probes[0] : nullptr;
-  a.snap_keys = snap_keys;
-  a.snap_amps = snap_amps;
-  a.snap_n = snap_n;
-  a.snap_stride = snap_stride;
   a.stats = k->stats;
   return a;
 }
 
+// A tape to record for the adjoint (out_pos with it), and whether the state keeps exact zeros.
+struct GateRun {
+  const GateTape* tape = nullptr;
+  bool keep_zeros = false;
+};
+
+// The gate sequence, in place (swcs_gates.cu).  Instances that share the device (batch mode 1, captured) and states
+// whose work arrays cannot be had run the rebuilding kernel (swcs_ansatz.cu), which needs half the memory.
 int run_gates(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, int64_t n_keep, bool reset,
-              uint64_t* snap_keys = nullptr, double* snap_amps = nullptr, long long* snap_n = nullptr,
-              int64_t snap_stride = 0, bool keep_zeros = false) {
+              const GateRun& run = GateRun()) {
+  if (!c->selhist.p) return fail(c, SWCS_ERR_CUDA, "gate kernel histograms not allocated");
+  Ctrl* k = ctrl(c);
+  const bool shared = c->opt_gate_threads != kAnsatzThreads;
+  int r = shared || c->max_state > kMaxInPlace ? 1 : ensure_gate_buffers(c);
+  if (r == SWCS_OK) {
+    GateArgs a{};
+    a.in_keys = (const uint64_t*)c->keys_a.p;
+    a.in_amps = (const double*)c->amps_a.p;
+    a.out_keys = (uint64_t*)c->keys_a.p;
+    a.out_amps = (double*)c->amps_a.p;
+    a.keys = (uint64_t*)c->keys_b.p;
+    a.amp[0] = (double*)c->amps_b.p;
+    a.amp[1] = (double*)c->amps_c.p;
+    a.cap = (uint32_t)(4 * c->max_state + 64);
+    a.tab = (uint64_t*)c->tab1.p;
+    a.tab_mask = 2 * c->tab_mask + 1;
+    a.plain = (IdxSlot*)c->tab0.p;
+    a.plain_mask = c->tab_mask;
+    a.low_keys = (uint64_t*)c->low_keys.p;
+    a.low_amps = (double*)c->low_amps.p;
+    a.low_rec = (uint32_t*)c->low_rec.p;
+    a.cap_low = (uint32_t)c->max_state;
+    a.ring = (uint32_t*)c->ring.p;
+    a.ring_mask = (uint32_t)(pow2_at_least(4 * (uint64_t)c->max_state + 64) - 1);
+    a.ops = d_ops;
+    a.cs = d_cs;
+    a.n_ops = n_ops;
+    a.n_keep = n_keep;
+    a.min_abs_bits = min_abs_bits(c, run.keep_zeros);
+    a.reset_to_hf = reset ? 1 : 0;
+    a.hf = (c->ne >= 64) ? ~0ull : ((1ull << c->ne) - 1ull);
+    a.n_state = &k->n_state;
+    a.ctr = k->gate_ctr;
+    a.hist = (unsigned*)c->selhist.p;
+    a.band = (unsigned*)c->band.p;
+    a.band_ent = (BandEntry*)c->band_slots.p;
+    a.band_slots = band_slots_for(c->max_state);
+    a.bar = &k->bar;
+    a.err = &k->err;
+    a.timeout_ns = c->opt_timeout_ns;
+    a.skip_arrive_block = c->opt_skip_arrive;
+    a.stats = k->stats;
+    a.probe_ctr = c->opt_count_probes ? &k->probes[0] : nullptr;
+    if (run.tape) {
+      a.tape = *run.tape;
+      a.out_pos = (uint32_t*)c->out_pos.p;
+    }
+    int nblocks = 0;
+    bool clustered = false;
+    gate_launch_shape(c, gate_blocks_per_sm(), &nblocks, &clustered);
+    if (!clustered) CK(cudaMemsetAsync(&k->bar, 0, sizeof(GridBar), c->st));  // barrier words must start at zero
+    CK(launch_k(c, kKAnsatz, [&] { return launch_gates(a, nblocks, clustered, c->st); }));
+    c->tab_cur = 0;
+    c->have_state = true;
+    c->n_state_host = -1;
+    return SWCS_OK;
+  }
+  if (run.tape || run.keep_zeros) return r == 1 ? fail(c, SWCS_ERR_OOM, "state too large for the adjoint") : r;
   const int gthreads = c->opt_gate_threads;
   const int bps = ansatz_blocks_per_sm(gthreads);
   if (bps <= 0) return fail(c, SWCS_ERR_NO_DEVICE, "ansatz kernel cannot be resident on this device");
-  if (!c->selhist.p) return fail(c, SWCS_ERR_CUDA, "gate kernel histograms not allocated");
-  const AnsatzArgs a = gate_args(c, d_ops, d_cs, n_ops, n_keep, reset, snap_keys, snap_amps, snap_n, snap_stride,
-                                 keep_zeros);
-  Ctrl* k = ctrl(c);
-  // barrier words must start at zero
+  const AnsatzArgs a = gate_args(c, d_ops, d_cs, n_ops, n_keep, reset);
   CK(cudaMemsetAsync(&k->bar, 0, sizeof(GridBar), c->st));
   int nblocks = c->nsm * bps;
   if (c->opt_gate_blocks > 0) {
@@ -928,8 +1036,9 @@ int swcs_destroy(swcs_ctx* c) {
                     &c->rank_tab, &c->atab,
                     &c->gid_of, &c->gcount, &c->goff, &c->gfill, &c->gkey, &c->gamp, &c->grank, &c->rows,
                     &c->rbeta, &c->gab, &c->kab, &c->gorig,
-                    &c->ck_keys, &c->ck_amps, &c->ck_n, &c->sn_keys, &c->sn_amps, &c->sn_n, &c->sigma, &c->nu0,
-                    &c->nu1, &c->atab0, &c->atab1, &c->dth, &c->pool_dev, &c->selbits, &c->feat,
+                    &c->ck_keys, &c->ck_amps, &c->ck_n, &c->tp_pos, &c->tp_x, &c->tp_drop, &c->tp_start, &c->sigma,
+                    &c->nu0, &c->nu1, &c->atab0, &c->dth, &c->amps_c, &c->low_keys, &c->low_amps, &c->low_rec, &c->ring,
+                    &c->out_pos, &c->band, &c->band_slots, &c->pool_dev, &c->selbits, &c->feat,
                     &c->ypred, &c->topk_hist, &c->topk_ctl, &c->occ, &c->prb, &c->ab_cnt, &c->ab_list,
                     &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items,
                     &c->rdm_tab, &c->rdm_work, &c->rdm_gamma};
@@ -1630,6 +1739,9 @@ int swcs_set_option(swcs_ctx* c, const char* name, int64_t value) {
     if (value != 128 && value != 256 && value != 512 && value != 1024)
       return fail(c, SWCS_ERR_INVALID_ARG, "threads must be 128, 256, 512 or 1024");
     c->opt_threads = (int)value;
+  } else if (k == "adjoint_tape_mb") {
+    if (value < 0) return fail(c, SWCS_ERR_INVALID_ARG, "adjoint_tape_mb must be >= 0");
+    c->opt_tape_mb = value;
   } else if (k == "pairs") {
     if (value < -1 || value > 1) return fail(c, SWCS_ERR_INVALID_ARG, "pairs must be -1, 0 or 1");
     c->opt_pairs = (int)value;
@@ -1685,19 +1797,51 @@ int swcs_energy_grad(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, i
   if (r) return r;
   if (n_ops <= 0 || !h_ops || !h_theta) return fail(c, SWCS_ERR_INVALID_ARG, "energy_grad needs at least one gate");
   if ((r = validate_ops(c, h_ops, n_ops))) return r;
-  const int ck = ckpt_every > 0 ? ckpt_every : 20;
-  const int ncp = (n_ops + ck - 1) / ck;
   const int64_t ms = max_state_for(c, n_keep, n_ops, 1);
-  if (ms > ((int64_t)1 << 31)) return fail(c, SWCS_ERR_INVALID_ARG, "state bound too large: give n_keep");
-  if ((r = ensure_state_buffers(c, ms))) return r;
-  const int64_t stride = ms + 64;
+  if (ms > kMaxInPlace) return fail(c, SWCS_ERR_INVALID_ARG, "state bound too large: give n_keep");
+  if ((r = ensure_state_buffers(c, ms)) || (r = ensure_gate_buffers(c))) return r;
+  const int64_t stride = c->max_state + 64, np = 4 * c->max_state + 64;
+  if ((r = ensure(c, c->sigma, (size_t)stride * 8)) || (r = ensure(c, c->nu0, (size_t)np * 8)) ||
+      (r = ensure(c, c->out_pos, (size_t)stride * 4)) || (r = ensure(c, c->dth, (size_t)n_ops * 8)) ||
+      (r = ensure(c, c->tp_start, (size_t)2 * (n_ops + 1) * 8)))
+    return r;
+  // The tape takes at most a block and a drop per determinant and gate.  Where that fits for all gates there are no
+  // checkpoints and no replays; else segments of ckpt_every gates, halved until their tape can be had.
+  GateTape tape{};
+  int ck = n_ops;
+  {
+    const size_t per_gate = (size_t)c->max_state * (sizeof(uint2) + sizeof(double2) + sizeof(uint32_t));
+    size_t limit = (size_t)c->opt_tape_mb << 20;
+    if (limit == 0 && c->tp_x.bytes < (size_t)n_ops * c->max_state * sizeof(double2)) {
+      size_t free_b = 0, total_b = 0;
+      CK(cudaMemGetInfo(&free_b, &total_b));
+      limit = free_b / 8;
+    } else if (limit == 0) {
+      limit = ~(size_t)0;  // held already
+    }
+    if ((size_t)n_ops * per_gate > limit || (int64_t)n_ops * c->max_state >= ((int64_t)1 << 31))
+      ck = std::min(n_ops, ckpt_every > 0 ? ckpt_every : 20);
+    for (;; ck = (ck + 1) / 2) {
+      const size_t cap = (size_t)ck * c->max_state;
+      const bool fits = cap < ((size_t)1 << 31) && !ensure(c, c->tp_pos, cap * sizeof(uint2)) &&
+                        !ensure(c, c->tp_x, cap * sizeof(double2)) && !ensure(c, c->tp_drop, cap * sizeof(uint32_t));
+      if (fits) {
+        tape.cap = tape.drop_cap = cap;
+        break;
+      }
+      if (ck == 1) return fail(c, SWCS_ERR_OOM, "tape of one gate does not fit");
+    }
+    tape.pos = (uint2*)c->tp_pos.p;
+    tape.x = (double2*)c->tp_x.p;
+    tape.drop = (uint32_t*)c->tp_drop.p;
+    tape.start = (unsigned long long*)c->tp_start.p;
+  }
+  const int ncp = (n_ops + ck - 1) / ck;
   const uint64_t tcap = c->tab_mask + 1;
-  if ((r = ensure(c, c->ck_keys, (size_t)(ncp + 1) * stride * 8)) || (r = ensure(c, c->ck_amps, (size_t)(ncp + 1) * stride * 8)) ||
-      (r = ensure(c, c->ck_n, (size_t)(ncp + 1) * 8)) || (r = ensure(c, c->sn_keys, (size_t)ck * stride * 8)) ||
-      (r = ensure(c, c->sn_amps, (size_t)ck * stride * 8)) || (r = ensure(c, c->sn_n, (size_t)ck * 8)) ||
-      (r = ensure(c, c->sigma, (size_t)stride * 8)) || (r = ensure(c, c->nu0, (size_t)stride * 8)) ||
-      (r = ensure(c, c->nu1, (size_t)stride * 8)) || (r = ensure(c, c->atab0, tcap * sizeof(IdxSlot))) ||
-      (r = ensure(c, c->atab1, tcap * sizeof(IdxSlot))) || (r = ensure(c, c->dth, (size_t)n_ops * 8)))
+  if (ncp > 1 &&
+      ((r = ensure(c, c->ck_keys, (size_t)(ncp + 1) * stride * 8)) || (r = ensure(c, c->ck_amps, (size_t)(ncp + 1) * stride * 8)) ||
+       (r = ensure(c, c->ck_n, (size_t)(ncp + 1) * 8)) || (r = ensure(c, c->nu1, (size_t)np * 8)) ||
+       (r = ensure(c, c->atab0, tcap * sizeof(IdxSlot)))))
     return r;
   if ((r = upload_ops(c, h_ops, h_theta, n_ops))) return r;
   Ctrl* k = ctrl(c);
@@ -1706,114 +1850,96 @@ int swcs_energy_grad(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, i
   long long* ckn = (long long*)c->ck_n.p;
   const uint8_t* dops = (const uint8_t*)c->ops_dev.p;
   const double* dcs = (const double*)c->cs_dev.p;
+  const size_t sbytes = (size_t)c->max_state * 8;
   auto save_slot = [&](int slot) -> int {
-    CK(cudaMemcpyAsync(ckk + (size_t)slot * stride, c->keys_a.p, stride * 8, cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemcpyAsync(cka + (size_t)slot * stride, c->amps_a.p, stride * 8, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpyAsync(ckk + (size_t)slot * stride, c->keys_a.p, sbytes, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpyAsync(cka + (size_t)slot * stride, c->amps_a.p, sbytes, cudaMemcpyDeviceToDevice, c->st));
     CK(cudaMemcpyAsync(ckn + slot, &k->n_state, 8, cudaMemcpyDeviceToDevice, c->st));
     return SWCS_OK;
   };
   auto load_slot = [&](int slot) -> int {
-    CK(cudaMemcpyAsync(c->keys_a.p, ckk + (size_t)slot * stride, stride * 8, cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemcpyAsync(c->amps_a.p, cka + (size_t)slot * stride, stride * 8, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpyAsync(c->keys_a.p, ckk + (size_t)slot * stride, sbytes, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpyAsync(c->amps_a.p, cka + (size_t)slot * stride, sbytes, cudaMemcpyDeviceToDevice, c->st));
     CK(cudaMemcpyAsync(&k->n_state, ckn + slot, 8, cudaMemcpyDeviceToDevice, c->st));
     return SWCS_OK;
   };
-  // ---- forward with a checkpoint before every segment and after the last gate
-  {
-    const uint64_t hf = (c->ne >= 64) ? ~0ull : ((1ull << c->ne) - 1ull);
-    const double one = 1.0;
-    const long long n1 = 1;
-    CK(cudaMemcpyAsync(ckk, &hf, 8, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(cka, &one, 8, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(ckn, &n1, 8, cudaMemcpyHostToDevice, c->st));
-    CK(cudaMemcpyAsync(&k->n_state, &n1, 8, cudaMemcpyHostToDevice, c->st));
-    CK(cudaStreamSynchronize(c->st));  // host staging above
-  }
+  GateRun plain, taped;
+  plain.keep_zeros = taped.keep_zeros = true;
+  taped.tape = &tape;
+  // ---- forward: a checkpoint before every segment but the first (it starts from the reference), the last one taped
   for (int seg = 0; seg < ncp; ++seg) {
     const int g0 = seg * ck, g1 = std::min(n_ops, g0 + ck);
     if (seg > 0 && (r = save_slot(seg))) return r;
-    if ((r = run_gates(c, dops + 5 * g0, dcs + 2 * g0, g1 - g0, n_keep, seg == 0, nullptr, nullptr, nullptr, 0, true)))
-      return r;
+    if ((r = run_gates(c, dops + 5 * g0, dcs + 2 * g0, g1 - g0, n_keep, seg == 0, seg == ncp - 1 ? taped : plain))) return r;
   }
-  if ((r = save_slot(ncp))) return r;
-  c->have_state = true;
+  if (ncp > 1 && (r = save_slot(ncp))) return r;
   if ((r = need_nonempty(c))) return r;
   // ---- energy, sigma and nu_M = P_M (H - E) psi_M on the final state
-  CK(cudaMemsetAsync(k->acc, 0, 16, c->st));
   const int nblk = c->nsm * sigma_blocks_per_sm();
-  c->have_state = true;
   if ((r = energy_rows(c, (double*)c->sigma.p)) == 1) {
     CK(cudaMemsetAsync(k->acc, 0, 16, c->st));
     CK(launch_k(c, kKEnergy, [&] { return launch_energy_sigma(ham_dev(c), state_dev(c), k->acc, (double*)c->sigma.p, nblk, c->st); }));
   } else if (r) {
     return r;
   }
-  IdxSlot* atab[2] = {(IdxSlot*)c->atab0.p, (IdxSlot*)c->atab1.p};
   double* nu[2] = {(double*)c->nu0.p, (double*)c->nu1.p};
-  CK(launch_k(c, kKOther, [&] { return launch_nu_init((const double*)c->amps_a.p, (const double*)c->sigma.p, &k->n_state, k->acc, nu[0], c->st); }));
-  CK(launch_k(c, kKOther, [&] { return launch_build_index(ckk + (size_t)ncp * stride, ckn + ncp, atab[0], tcap - 1, c->st); }));
+  CK(cudaMemsetAsync(nu[0], 0, (size_t)np * 8, c->st));
+  CK(cudaMemsetAsync(&k->zeros, 0, 8, c->st));
+  CK(launch_k(c, kKOther, [&] {
+    return launch_nu_final((const double*)c->amps_a.p, (const double*)c->sigma.p, (const uint32_t*)c->out_pos.p, &k->n_state,
+                           k->acc, nu[0], &k->zeros, c->st);
+  }));
   CK(cudaMemsetAsync(c->dth.p, 0, (size_t)n_ops * 8, c->st));
-  int cur = 0;
-  const int adj_blocks = c->nsm * 8;
-  // ---- backward, one segment at a time
+  // ---- backward, one segment at a time: the segment's tape again, nu brought to its last positions by key
+  int cur = 0, nblocks = 0;
+  bool clustered = false;
+  gate_launch_shape(c, back_blocks_per_sm(), &nblocks, &clustered);
   for (int seg = ncp - 1; seg >= 0; --seg) {
     const int g0 = seg * ck, g1 = std::min(n_ops, g0 + ck);
-    if ((r = load_slot(seg))) return r;
-    if (g1 - g0 > 1) {
-      if ((r = run_gates(c, dops + 5 * g0, dcs + 2 * g0, g1 - g0 - 1, n_keep, false, (uint64_t*)c->sn_keys.p,
-                         (double*)c->sn_amps.p, (long long*)c->sn_n.p, stride, true)))
-        return r;
-    }
-    for (int g = g1 - 1; g >= g0; --g) {
-      const uint64_t* keys_g;
-      const double* amps_g;
-      const long long* n_g;
-      if (g == g0) {
-        keys_g = ckk + (size_t)seg * stride;
-        amps_g = cka + (size_t)seg * stride;
-        n_g = ckn + seg;
-      } else {
-        keys_g = (const uint64_t*)c->sn_keys.p + (size_t)(g - g0 - 1) * stride;
-        amps_g = (const double*)c->sn_amps.p + (size_t)(g - g0 - 1) * stride;
-        n_g = (const long long*)c->sn_n.p + (g - g0 - 1);
-      }
-      CK(launch_k(c, kKOther, [&] { return launch_build_index(keys_g, n_g, atab[cur ^ 1], tcap - 1, c->st); }));
-      AdjArgs a;
-      a.op = dops + 5 * g;
-      a.cs = dcs + 2 * g;
-      a.keys = keys_g;
-      a.amps = amps_g;
-      a.n = n_g;
-      a.tab = atab[cur ^ 1];
-      a.mask = tcap - 1;
-      a.tab_nu = atab[cur];
-      a.mask_nu = tcap - 1;
-      a.nu_in = nu[cur];
-      a.nu_out = nu[cur ^ 1];
-      a.dtheta = (double*)c->dth.p + g;
-      CK(launch_k(c, kKAdjoint, [&] { return launch_adjoint_gate(a, adj_blocks, c->st); }));
+    if (seg < ncp - 1) {
+      if (seg > 0 && (r = load_slot(seg))) return r;
+      if ((r = run_gates(c, dops + 5 * g0, dcs + 2 * g0, g1 - g0, n_keep, seg == 0, taped))) return r;
+      CK(launch_k(c, kKOther, [&] {
+        return launch_build_index(ckk + (size_t)(seg + 1) * stride, ckn + seg + 1, (IdxSlot*)c->atab0.p, tcap - 1, c->st);
+      }));
+      CK(cudaMemsetAsync(nu[cur ^ 1], 0, (size_t)np * 8, c->st));
+      CK(launch_k(c, kKOther, [&] {
+        return launch_nu_realign((const uint64_t*)c->keys_a.p, (const uint32_t*)c->out_pos.p, &k->n_state,
+                                 (const IdxSlot*)c->atab0.p, tcap - 1, nu[cur], nu[cur ^ 1], c->st);
+      }));
       cur ^= 1;
     }
+    BackArgs a{};
+    a.tape = tape;
+    a.cs = dcs + 2 * g0;
+    a.n_ops = g1 - g0;
+    a.nu = nu[cur];
+    a.dtheta = (double*)c->dth.p + g0;
+    a.bar = &k->bar;
+    a.err = &k->err;
+    a.timeout_ns = c->opt_timeout_ns;
+    if (!clustered) CK(cudaMemsetAsync(&k->bar, 0, sizeof(GridBar), c->st));
+    CK(launch_k(c, kKAdjoint, [&] { return launch_back(a, nblocks, clustered, c->st); }));
   }
   CK(launch_k(c, kKOther, [&] { return launch_scale_dtheta((double*)c->dth.p, n_ops, k->acc, c->st); }));
   CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(k->acc, k->eout, c->st); }));
-  // leave psi_M as the context's state (an identity pass rebuilds the index
-  // table and drops the zero amplitudes the projectors kept)
-  if ((r = load_slot(ncp))) return r;
-  {
-    const uint8_t id[5] = {0, 0, 0, 0, 0};
-    if ((r = ensure(c, c->gsub, 16))) return r;
-    CK(cudaMemcpyAsync(c->gsub.p, id, 5, cudaMemcpyHostToDevice, c->st));
-    const double z[2] = {1.0, 0.0};
-    if ((r = ensure(c, c->subset_dev, 16))) return r;
-    CK(cudaMemcpyAsync(c->subset_dev.p, z, 16, cudaMemcpyHostToDevice, c->st));
-    if ((r = run_gates(c, (const uint8_t*)c->gsub.p, (const double*)c->subset_dev.p, 1, 0, false))) return r;
-  }
+  if (ncp > 1 && (r = load_slot(ncp))) return r;
   double out[2];
+  unsigned long long zeros = 0;
   CK(cudaMemcpyAsync(out, k->eout, 16, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaMemcpyAsync(&zeros, &k->zeros, 8, cudaMemcpyDeviceToHost, c->st));
   if (h_dtheta_out) CK(cudaMemcpyAsync(h_dtheta_out, c->dth.p, (size_t)n_ops * 8, cudaMemcpyDeviceToHost, c->st));
   if ((r = check_device(c, "swcs_energy_grad"))) return r;
   if (h_e_out) *h_e_out = out[0];
+  // leave psi_M as the context's state: an identity pass rebuilds the index after replays and drops the zero
+  // amplitudes that the projectors kept
+  if (ncp > 1 || zeros) {
+    const uint8_t id[5] = {0, 0, 0, 0, 0};
+    const double z = 0.0;
+    if ((r = upload_ops(c, id, &z, 1))) return r;
+    if ((r = run_gates(c, (const uint8_t*)c->ops_dev.p, (const double*)c->cs_dev.p, 1, 0, false))) return r;
+    if ((r = check_device(c, "swcs_energy_grad"))) return r;
+  }
   return SWCS_OK;
 }
 
@@ -1972,8 +2098,7 @@ int batch_build_persistent(swcs_batch* b, int tile, int occ, int hash_factor) {
       return bfail(b, r, "batch: " + c->err);
     const int packed = c->NB <= (1 << 21) && m <= 32 ? 1 : 0;
     BatchInst& I = hi[i];
-    I.ga = gate_args(c, (const uint8_t*)c->ops_dev.p, (const double*)c->cs_dev.p, b->n_ops[i], b->n_keep[i], true,
-                     nullptr, nullptr, nullptr, 0, false);
+    I.ga = gate_args(c, (const uint8_t*)c->ops_dev.p, (const double*)c->cs_dev.p, b->n_ops[i], b->n_keep[i], true);
     I.gr = group_args(c, acap);
     I.ra = row_args(c, I.gr, (double*)c->gdev.p, max_s, max_d, twords, packed);
     I.n_ops = b->n_ops[i];

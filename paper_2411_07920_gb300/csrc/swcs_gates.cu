@@ -1,0 +1,985 @@
+// The gate sequence of the ansatz in one launch, every determinant at a fixed
+// position for as long as it lives.
+//
+// A gate rotates two-determinant blocks (Eqs. 2-3) and the truncation drops
+// the smallest amplitudes (Sec. II.B).  Most determinants of a large state are
+// outside every block, few new ones survive the truncation, and few old ones
+// are dropped, so nothing is rebuilt: one pass over the positions per gate
+//   - drops what the previous truncation cut (the cut is known by then: no
+//     pass of its own), handing the position on to be reused two gates later;
+//   - rotates the blocks from one amplitude array into the other (the lower
+//     member writes both), a partner that is not in the state taking a free
+//     position and an index slot;
+//   - counts |c| in narrow bins around the previous gate's cut, keeping the
+//     few entries of each bin, and the number of larger ones.
+// After one barrier every CTA finds the bin that holds the new cut and, among
+// its entries, the cut itself, exactly.  Only where the cut leaves the band (or
+// its bin overflows, or there was no cut before) does the general radix select
+// over 12-bit digits follow, a pass over the amplitudes and a barrier each.  A
+// new partner with |c| below half the previous cut is put aside instead of into
+// the state; when the new cut turns out to be lower than that (rare: rotations
+// must have shrunk the bulk of the kept amplitudes), those that are kept are
+// added by a pass of their own.
+//
+// Amplitudes are computed as in swcs_ansatz.cu (at most two separately rounded
+// products each), and the cut is exact including ties, so states are
+// bit-identical to any sequential evaluation.
+//
+// Per gate (rebuilding kernel of swcs_ansatz.cu before): 50 us at 10^6
+// determinants (73 us), 15 us at 33,333 (22.5 us), 9 us at 38,701 without a cut
+// (14.7 us), 6 us at a few hundred (10 us); the adjoint's backward pass 7.8 us a
+// gate at 10^6 (77 us with index builds).  A gate is a chain of dependent L2
+// accesses -- amplitude and key, index sector, partner, places in the lists,
+// index slot -- and a barrier, about 0.6 us each, once per batch of 2,048
+// positions and CTA; memory traffic is a fifth of the time at 10^6.
+//
+// Up to 16,384 determinants the CTAs form one thread-block cluster, with its
+// hardware barrier (0.7 us) and the counters in the first CTA's shared memory;
+// above, a grid of one CTA per 512 determinants with a bounded barrier (2.3 us)
+// beats 16 CTAs that work several batches one after another (13.9 + 4 us
+// against 7.6 + 3 at 33,333).  With a tape (adjoint) the pass also records each block's
+// positions and amplitudes and each dropped position; the backward pass then
+// needs neither index nor snapshot, only these lists and nu by position.
+#include <cooperative_groups.h>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "swcs_device.cuh"
+#include "swcs_gates.h"
+#include "swcs_kernels.h"
+#include "swcs_select.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace swcs {
+
+namespace {
+
+// Bit patterns of dead positions (NaNs no arithmetic produces): dropped in the pass before, free.
+constexpr unsigned long long kDead1 = 0x7FF8DEAD00000001ull, kDead2 = 0x7FF8DEAD00000002ull;
+
+enum { kGcExtra = 0, kGcLow, kGcZero, kGcPush, kGcRec, kGcDrop, kGcAbove };
+
+__device__ __forceinline__ unsigned long long bits_of(double c) { return (unsigned long long)__double_as_longlong(c); }
+__device__ __forceinline__ bool dead(unsigned long long b) { return b == kDead1 || b == kDead2; }
+
+// A distinct place from a counter in shared memory for every lane with pred; all 32 lanes call it.
+__device__ __forceinline__ unsigned claim(unsigned* ctr, bool pred) {
+  const unsigned b = __ballot_sync(0xffffffffu, pred);
+  if (!b) return 0;
+  const int lane = threadIdx.x & 31;
+  unsigned base = 0;
+  if (lane == 0) base = atomicAdd(ctr, (unsigned)__popc(b));
+  return __shfl_sync(0xffffffffu, base, 0) + __popc(b & ((1u << lane) - 1u));
+}
+
+// Barrier of the launch's CTAs: a cluster's hardware barrier, or a monotonic counter (bar->count; `round` counts the
+// barriers) polled for at most timeout_ns, after which (or on another CTA's error) every CTA leaves.
+template <bool CLUSTER>
+__device__ __forceinline__ bool gate_sync(GridBar* bar, unsigned nblocks, unsigned& round, int* err, uint64_t timeout_ns) {
+  if (CLUSTER) {
+    if (nblocks == 1) __syncthreads();
+    else cg::this_cluster().sync();
+    return true;  // a cluster's CTAs leave together, at the end
+  }
+  __shared__ int s_ok;
+  __syncthreads();
+  ++round;
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    const unsigned target = round * nblocks;
+    __threadfence();
+    atomicAdd(&bar->count, 1u);
+    uint64_t t0 = 0;
+    for (unsigned spins = 1; (int)(ld_acquire_u32(&bar->count) - target) < 0; ++spins) {
+      if ((spins & 255u) == 0) {
+        if (ld_acquire_i32(err) != 0) { ok = 0; break; }
+        const uint64_t t = globaltimer_ns();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > timeout_ns) { set_error(err, kDevTimeout); ok = 0; break; }
+      }
+    }
+    __threadfence();
+    if (ok && ld_acquire_i32(err) != 0) ok = 0;
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// The index: linear probing over 8-byte slots of epoch (16 bits), fingerprint of the key (16), position (32).  A slot
+// of another epoch is empty.  Probes read whole 32-byte sectors, four slots at a time, and a determinant's key only
+// where the fingerprint fits: dropped determinants leave their slots behind, so runs get long, and a chain of
+// dependent loads per slot made the slowest warp of a batch wait for 15 us.
+__device__ __forceinline__ unsigned long long slot_head(uint32_t ep, uint64_t hash) {
+  return ((unsigned long long)ep << 48) | ((hash >> 48) << 32);
+}
+
+struct Probe {
+  uint64_t slot;            // where the search ended: the key's slot, or an empty one
+  unsigned long long word;  // and what it held
+};
+
+// Position of key among the state's determinants (-1: absent) and its amplitude.  Slots of this pass's own new
+// determinants point at or above limit, or at reused positions, whose old amplitude is a dead one; so a match that is
+// not alive does not end the search.
+// s0, s1: the sector of the home slot.
+template <class Alive>
+__device__ __forceinline__ int64_t find_key(const uint64_t* tab, uint64_t mask, const uint64_t* keys, const double* A,
+                                            uint64_t key, uint64_t hash, ulonglong2 s0, ulonglong2 s1, uint32_t ep,
+                                            uint32_t limit, double* amp, unsigned* probes, Probe* at, Alive&& alive) {
+  const unsigned long long want = slot_head(ep, hash) >> 32;
+  uint64_t base = hash & mask & ~3ull;
+  int first = (int)(hash & mask & 3ull);
+  at->word = ~0ull;
+  at->slot = base + first;
+  for (uint64_t n = 0; n <= mask; n += 4) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const unsigned long long w = q == 0 ? s0.x : q == 1 ? s0.y : q == 2 ? s1.x : s1.y;
+      if (q < first) continue;
+      *probes += 1u;
+      if ((uint32_t)(w >> 48) != ep) {
+        at->slot = base + q;
+        at->word = w;
+        return -1;
+      }
+      const uint32_t p = (uint32_t)w;
+      if ((w >> 32) == want && p < limit) {
+        const uint64_t k = __ldcg((const unsigned long long*)&keys[p]);
+        const double c = __ldcg(&A[p]);
+        if (k == key && alive(c)) {
+          *amp = c;
+          return (int64_t)p;
+        }
+      }
+    }
+    first = 0;
+    base = (base + 4) & mask;
+    s0 = __ldcg((const ulonglong2*)&tab[base]);
+    s1 = __ldcg((const ulonglong2*)&tab[base + 2]);
+  }
+  return -1;
+}
+
+// Inserts a key that is not in the index.
+__device__ __forceinline__ bool put_key(uint64_t* tab, uint64_t mask, uint64_t hash, uint32_t pos, uint32_t ep) {
+  const unsigned long long mine = slot_head(ep, hash) | pos;
+  uint64_t s = hash & mask;
+  for (uint64_t n = 0; n <= mask; ++n) {
+    unsigned long long* w = (unsigned long long*)&tab[s];
+    const unsigned long long old = __ldcg(w);
+    if ((uint32_t)(old >> 48) != ep && atomicCAS(w, old, mine) == old) return true;
+    s = (s + 1) & mask;
+  }
+  return false;
+}
+
+constexpr int kU = 2;                       // positions a thread works on at a time, their loads issued together
+constexpr int kList = kU * kGateThreads;    // entries of a batch's lists: at most one per position
+constexpr int kBandList = kList;            // amplitudes inside the band (more go to the bins one by one)
+
+// What a batch of positions leaves to be done, collected in shared memory so that a CTA takes its places in the
+// global lists with one atomic each and works the entries off side by side: a chain of global atomics per warp
+// (positions, free ring, index slot, bins) cost 10 us a batch.
+struct GateLists {
+  uint64_t* partner;     // blocks whose partner is not in the state (with a tape: every block)
+  double *extra, *c, *xm;
+  unsigned long long* word;  // index slot where the partner's search ended, as it was read
+  uint32_t *slot, *pos, *mate, *info, *rank;
+  BandEntry* band;
+  uint32_t *push, *drop;
+};
+enum : uint32_t { kHigh = 1u, kLow = 2u, kLower = 4u, kPhase = 8u };
+enum { kCList = 0, kCHigh, kCLow, kCBand, kCPush, kCDrop, kCZero, kCAbove, kCN };
+
+constexpr size_t kGateSmem = (size_t)kList * (8 * 5 + 4 * 5 + 4 * 2) + (size_t)kBandList * sizeof(BandEntry);
+
+__device__ __forceinline__ GateLists gate_lists(unsigned char* sm) {
+  GateLists L;
+  L.band = (BandEntry*)sm;
+  L.partner = (uint64_t*)(L.band + kBandList);
+  L.extra = (double*)(L.partner + kList);
+  L.c = L.extra + kList;
+  L.xm = L.c + kList;
+  L.word = (unsigned long long*)(L.xm + kList);
+  L.slot = (uint32_t*)(L.word + kList);
+  L.pos = L.slot + kList;
+  L.mate = L.pos + kList;
+  L.info = L.mate + kList;
+  L.rank = L.info + kList;
+  L.push = L.rank + kList;
+  L.drop = L.push + kList;
+  return L;
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kGateThreads) gates_kernel(GateArgs a) {
+  extern __shared__ __align__(16) unsigned char gate_dyn[];
+  __shared__ SelState sel;
+  __shared__ unsigned s_h0[kBins];
+  __shared__ long long s_scan[32];
+  __shared__ unsigned long long s_base;
+  __shared__ long long s_n;
+  __shared__ unsigned s_cnt[kCN], s_grp[kBandGroups];
+  __shared__ unsigned long long s_ctr[3 * kGateCtrN];
+  __shared__ unsigned long long s_at[kCN];
+  const GateLists L = gate_lists(gate_dyn);
+  const unsigned nb = gridDim.x;
+  const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, gstride = nb * blockDim.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned n_lookups = 0, n_slots = 0, round = 0;
+  const bool taped = a.tape.pos != nullptr;
+  // the gates' counters: in the first CTA's shared memory where the CTAs form a cluster
+  unsigned long long* ctr_all = a.ctr;
+  if (CLUSTER) ctr_all = nb == 1 ? s_ctr : cg::this_cluster().map_shared_rank(s_ctr, 0);
+
+  // ---------------------------------------------------------------- tables cleared, the input at positions 0 .. n - 1
+  if (threadIdx.x == 0) s_n = a.reset_to_hf ? 1 : *a.n_state;
+  __syncthreads();
+  const uint32_t n_in = (uint32_t)s_n;
+  for (uint64_t i = gtid; i <= a.tab_mask; i += gstride) a.tab[i] = 0;  // epoch 0: no build
+  for (uint64_t i = gtid; i <= a.plain_mask; i += gstride) {
+    a.plain[i].key = kEmpty;
+    a.plain[i].idx = 0;
+  }
+  if (a.n_keep > 0)
+    for (uint32_t i = gtid; i < 3 * kBandWords; i += gstride) a.band[i] = 0;
+  if (gtid < 3 * kGateCtrN) (CLUSTER ? s_ctr : a.ctr)[gtid] = 0;  // the first CTA's threads
+  if (gtid == 0) a.ctr[3 * kGateCtrN] = 0;
+  if (a.reset_to_hf) {
+    if (gtid == 0) {
+      a.keys[0] = a.hf;
+      a.amp[0][0] = 1.0;
+    }
+  } else {
+    for (uint32_t i = gtid; i < n_in; i += gstride) {
+      a.keys[i] = a.in_keys[i];
+      a.amp[0][i] = a.in_amps[i];
+    }
+  }
+  if (!CLUSTER && (int)blockIdx.x == a.skip_arrive_block) return;  // test hook: never arrives, the others' waits run out
+  if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+  uint32_t ep = 1;
+  for (uint32_t i = gtid; i < n_in; i += gstride)
+    if (!put_key(a.tab, a.tab_mask, mix64(a.keys[i]), i, ep)) set_error(a.err, kDevTableFull);
+  if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+
+  // the same in every CTA
+  uint32_t nt = n_in;                     // positions in use
+  uint64_t live = n_in;                   // determinants of the state
+  uint64_t used = n_in;                   // index slots taken since the build
+  unsigned long long head = 0, tail = 0;  // free positions in the ring
+  unsigned long long rec0 = 0, drop0 = 0;  // tape entries of the gates before
+  SelState cut{};                         // what the last truncation keeps
+  int cur = 0;
+  int dirty0 = 0, dirty1 = 0, dirty2 = 0;  // whether each band set has counts, this gate's first
+  if (threadIdx.x < kCN) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x < kBandGroups) s_grp[threadIdx.x] = 0;
+  __syncthreads();
+  // ---------------------------------------------------------------- the gates
+  for (int g = 0; g < a.n_ops; ++g) {
+    const GateOp op = decode_op(a.ops + 5 * g);
+    const double cs = a.cs[2 * g], sn = a.cs[2 * g + 1];
+    unsigned long long* ctr = ctr_all + (g % 3) * kGateCtrN;
+    unsigned* band = a.band + (size_t)(g % 3) * kBandWords;
+    BandEntry* slots = a.band_ent + (size_t)(g % 3) * kBandBins * a.band_slots;
+    double* A = a.amp[cur];
+    double* B = a.amp[cur ^ 1];
+    if (used + live > (a.tab_mask + 1) / 4 * 3) {  // slots of dropped determinants fill the index: build it anew
+      if (++ep > 0xFFFFu) {  // epochs used up: every slot cleared once
+        for (uint64_t i = gtid; i <= a.tab_mask; i += gstride) a.tab[i] = 0;
+        if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+        ep = 1;
+      }
+      for (uint32_t i = gtid; i < nt; i += gstride) {
+        const double c = __ldcg(&A[i]);
+        if (dead(bits_of(c))) continue;
+        const uint64_t d = __ldcg((const unsigned long long*)&a.keys[i]);
+        if (keep_entry(cut, d, c, a.min_abs_bits) && !put_key(a.tab, a.tab_mask, mix64(d), i, ep)) set_error(a.err, kDevTableFull);
+      }
+      if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+      used = live;
+    }
+    // partners below half the last cut are put aside (its exponent less one; never below the smallest normal)
+    const uint64_t filter = cut.mode && cut.prefix > (2ull << 52) ? cut.prefix - (1ull << 52) : 0ull;
+    const uint64_t mid = (cut.prefix >> kBandShift) << kBandShift, half = (uint64_t)(kBandBins / 2) << kBandShift;
+    const bool banded = cut.mode != 0 && a.n_keep > 0 && mid > half + a.min_abs_bits;
+    const uint64_t b_lo = mid - half, b_hi = mid + half;
+    {  // the next gate's counters and bins, last read two gates ago
+      unsigned long long* cn = ctr_all + ((g + 1) % 3) * kGateCtrN;
+      if (gtid < kGateCtrN) cn[gtid] = 0;
+      if (dirty1) {
+        unsigned* bn = a.band + (size_t)((g + 1) % 3) * kBandWords;
+        for (uint32_t i = gtid; i < kBandWords; i += gstride) bn[i] = 0;
+      }
+      dirty1 = 0;
+      if (banded) dirty0 = 1;
+    }
+    if (taped && gtid == 0) {
+      a.tape.start[2 * g] = rec0;
+      a.tape.start[2 * g + 1] = drop0;
+    }
+    unsigned above = 0;
+    bool left = false;  // this thread left something in the batch's lists
+    auto to_bin = [&](unsigned long long x, unsigned long long k) {
+      const uint32_t b = (uint32_t)((x - b_lo) >> kBandShift);
+      const unsigned q = atomicAdd(&band[b], 1u);
+      atomicAdd(&s_grp[b >> 7], 1u);
+      if (q < (unsigned)a.band_slots) slots[b * a.band_slots + q] = BandEntry{x, k};
+    };
+    auto tally = [&](uint64_t k, double c) {
+      if (!banded) return;
+      const uint64_t x = abs_bits(c);
+      if (x >= b_hi) {
+        ++above;
+      } else if (x >= b_lo) {
+        const cg::coalesced_group in = cg::coalesced_threads();
+        unsigned q = 0;
+        if (in.thread_rank() == 0) q = atomicAdd(&s_cnt[kCBand], in.size());
+        q = in.shfl(q, 0) + in.thread_rank();
+        left = true;
+        if (q < kBandList) L.band[q] = BandEntry{x, k};
+        else to_bin(x, k);
+      }
+    };
+    const unsigned long long n_free = tail - head;
+    // the k-th new determinant's position: a free one, else one at the end
+    auto place = [&](unsigned long long k, uint32_t nt0) -> uint32_t {
+      const unsigned long long p = k < n_free ? __ldcg(&a.ring[(head + k) & a.ring_mask]) : nt0 + (k - n_free);
+      if (p < a.cap) return (uint32_t)p;
+      set_error(a.err, kDevTableFull);  // cannot happen: see the buffers' sizes
+      return kNoPos;
+    };
+    const uint32_t nt_pass = nt;
+    auto alive_in = [&](uint64_t d, double c) { return !dead(bits_of(c)) && (g == 0 || keep_entry(cut, d, c, a.min_abs_bits)); };
+    for (uint32_t r0 = blockIdx.x * blockDim.x; r0 < nt_pass; r0 += kU * gstride) {  // the same rounds for the whole CTA
+      const uint32_t i0 = r0 + threadIdx.x;
+      double c[kU];
+      uint64_t d[kU], partner[kU];
+      ulonglong2 w0[kU], w1[kU];
+      int role[kU], sbit[kU];
+      unsigned push = 0, drop = 0, zero = 0, acts = 0;
+      left = false;
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const uint32_t i = i0 + u * gstride;
+        c[u] = i < nt_pass ? __ldcg(&A[i]) : __longlong_as_double((long long)kDead2);
+        d[u] = i < nt_pass ? __ldcg((const unsigned long long*)&a.keys[i]) : 0ull;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const uint32_t i = i0 + u * gstride;
+        const unsigned long long b = bits_of(c[u]);
+        role[u] = sbit[u] = 0;
+        partner[u] = 0;
+        if (b == kDead2) continue;
+        if (b == kDead1) {  // dropped in the last pass: free from the next gate on
+          A[i] = __longlong_as_double((long long)kDead2);
+          B[i] = __longlong_as_double((long long)kDead2);
+          push |= 1u << u;
+        } else if (!alive_in(d[u], c[u])) {
+          B[i] = __longlong_as_double((long long)kDead1);
+          drop |= 1u << u;
+        } else {
+          role[u] = gate_role(op, d[u], &partner[u], &sbit[u]);
+          if (role[u] == 0) {
+            B[i] = c[u];
+            if (abs_bits(c[u]) < a.min_abs_bits) ++zero;
+            tally(d[u], c[u]);
+          } else {
+            acts |= 1u << u;
+            const uint64_t s = mix64(partner[u]) & a.tab_mask & ~3ull;
+            w0[u] = __ldcg((const ulonglong2*)&a.tab[s]);
+            w1[u] = __ldcg((const ulonglong2*)&a.tab[s + 2]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const uint32_t i = i0 + u * gstride;
+        double extra = 0.0, xm = 0.0;
+        uint32_t mate = kNoPos, info = 0;
+        bool listed = false;
+        Probe at{0, 0};
+        if (acts >> u & 1u) {
+          ++n_lookups;
+          const int64_t j = find_key(a.tab, a.tab_mask, a.keys, A, partner[u], mix64(partner[u]), w0[u], w1[u], ep, nt_pass,
+                                     &xm, &n_slots, &at, [&](double x) { return alive_in(partner[u], x); });
+          const double t1 = __dmul_rn(c[u], cs), t2 = __dmul_rn(c[u], sn);
+          info = (role[u] > 0 ? kLower : 0u) | (sbit[u] ? kPhase : 0u);
+          if (j >= 0) {
+            if (role[u] > 0) {  // lower D writes both: c' = c cos - s sin c_U ; c'_U = c_U cos + s sin c
+              mate = (uint32_t)j;
+              const double lo = __dadd_rn(t1, apply_sign(__dmul_rn(xm, sn), !sbit[u]));
+              const double up = __dadd_rn(__dmul_rn(xm, cs), apply_sign(t2, sbit[u]));
+              B[i] = lo;
+              B[j] = up;
+              zero += (abs_bits(lo) < a.min_abs_bits) + (abs_bits(up) < a.min_abs_bits);
+              tally(d[u], lo);
+              tally(partner[u], up);
+              listed = taped;
+            }  // the upper member's block is its lower partner's work
+          } else {
+            B[i] = t1;
+            zero += abs_bits(t1) < a.min_abs_bits;
+            tally(d[u], t1);
+            extra = role[u] > 0 ? apply_sign(t2, sbit[u]) : apply_sign(t2, !sbit[u]);
+            if (abs_bits(extra) >= a.min_abs_bits) info |= abs_bits(extra) >= filter ? kHigh : kLow;
+            listed = taped || (info & (kHigh | kLow));
+          }
+        }
+        const unsigned q = claim(&s_cnt[kCList], listed);
+        const unsigned qh = claim(&s_cnt[kCHigh], listed && (info & kHigh)), ql = claim(&s_cnt[kCLow], listed && (info & kLow));
+        left |= listed;
+        if (listed) {
+          L.partner[q] = partner[u];
+          L.extra[q] = extra;
+          L.word[q] = at.word;
+          L.slot[q] = (uint32_t)at.slot;
+          L.info[q] = info;
+          L.rank[q] = info & kHigh ? qh : ql;
+          if (taped) {
+            L.c[q] = c[u];
+            L.xm[q] = xm;
+            L.pos[q] = i;
+            L.mate[q] = mate;
+          }
+        }
+        const unsigned qp = claim(&s_cnt[kCPush], push >> u & 1u);
+        if (push >> u & 1u) L.push[qp] = i;
+        if (taped) {
+          const unsigned qd = claim(&s_cnt[kCDrop], drop >> u & 1u);
+          if (drop >> u & 1u) L.drop[qd] = i;
+        }
+      }
+      if (__any_sync(0xffffffffu, zero)) {
+        zero = __reduce_add_sync(0xffffffffu, zero);
+        if (lane == 0) atomicAdd(&s_cnt[kCZero], zero);
+      }
+      // ---- the batch's lists
+      left |= push != 0 || (taped && drop != 0);
+      if (__syncthreads_or(left)) {
+        const unsigned n_list = s_cnt[kCList], n_band = min(s_cnt[kCBand], (unsigned)kBandList), n_push = s_cnt[kCPush];
+        const unsigned n_drop = s_cnt[kCDrop];
+        if (wid == 0 && lane < kCN) {  // one atomic per global list
+          const unsigned n = s_cnt[lane];
+          unsigned long long* to = lane == kCHigh ? &ctr[kGcExtra] : lane == kCLow ? &ctr[kGcLow] : lane == kCPush ? &ctr[kGcPush]
+                                 : lane == kCDrop ? &ctr[kGcDrop] : lane == kCList && taped ? &ctr[kGcRec] : nullptr;
+          if (to && n) s_at[lane] = atomicAdd(to, (unsigned long long)n);
+        }
+        for (unsigned q = threadIdx.x; q < n_band; q += blockDim.x) to_bin(L.band[q].x, L.band[q].key);
+        __syncthreads();
+        for (unsigned q = threadIdx.x; q < n_list; q += blockDim.x) {
+          const uint32_t info = L.info[q];
+          const uint64_t key = L.partner[q];
+          const double extra = L.extra[q];
+          uint32_t mate = taped ? L.mate[q] : kNoPos;
+          if (info & kHigh) {
+            const uint32_t p = place(s_at[kCHigh] + L.rank[q], nt_pass);
+            if (p != kNoPos) {
+              a.keys[p] = key;
+              B[p] = extra;
+              if (p >= nt_pass) A[p] = __longlong_as_double((long long)kDead2);
+              mate = p;
+              // the slot where the search ended, unless another new determinant has taken it meanwhile
+              const uint64_t hash = mix64(key);
+              const unsigned long long mine = slot_head(ep, hash) | p, was = L.word[q];
+              if (((uint32_t)(was >> 48) == ep || atomicCAS((unsigned long long*)&a.tab[L.slot[q]], was, mine) != was) &&
+                  !put_key(a.tab, a.tab_mask, hash, p, ep))
+                set_error(a.err, kDevTableFull);
+              if (banded) {
+                const uint64_t x = abs_bits(extra);
+                if (x >= b_hi) ++above;
+                else if (x >= b_lo) to_bin(x, key);
+              }
+            }
+          }
+          const unsigned long long rec = s_at[kCList] + q;
+          if (taped && rec0 + rec < a.tape.cap) {
+            const bool lo = info & kLower;
+            const uint32_t i = L.pos[q];
+            a.tape.pos[rec0 + rec] = make_uint2(((lo ? i : mate) & 0x7FFFFFFFu) | (info & kPhase ? 0x80000000u : 0u), lo ? mate : i);
+            a.tape.x[rec0 + rec] = lo ? make_double2(L.c[q], L.xm[q]) : make_double2(L.xm[q], L.c[q]);
+          }
+          if (info & kLow) {
+            const unsigned long long k = s_at[kCLow] + L.rank[q];
+            if (k < a.cap_low) {
+              a.low_keys[k] = key;
+              a.low_amps[k] = extra;
+              a.low_rec[k] = taped ? ((uint32_t)rec | (info & kLower ? 0x80000000u : 0u)) : 0u;
+            }
+          }
+        }
+        for (unsigned q = threadIdx.x; q < n_push; q += blockDim.x) a.ring[(tail + s_at[kCPush] + q) & a.ring_mask] = L.push[q];
+        for (unsigned q = threadIdx.x; q < n_drop; q += blockDim.x)
+          if (drop0 + s_at[kCDrop] + q < a.tape.drop_cap) a.tape.drop[drop0 + s_at[kCDrop] + q] = L.drop[q];
+        __syncthreads();
+        if (threadIdx.x < kCZero) s_cnt[threadIdx.x] = 0;  // (above and zeros run on to the end of the pass)
+        __syncthreads();
+      }
+    }
+    if (__any_sync(0xffffffffu, above)) {
+      above = __reduce_add_sync(0xffffffffu, above);
+      if (lane == 0) atomicAdd(&s_cnt[kCAbove], above);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (s_cnt[kCAbove]) atomicAdd(&ctr[kGcAbove], (unsigned long long)s_cnt[kCAbove]);
+      if (s_cnt[kCZero]) atomicAdd(&ctr[kGcZero], (unsigned long long)s_cnt[kCZero]);
+      s_cnt[kCAbove] = s_cnt[kCZero] = 0;
+    }
+    if (banded && threadIdx.x < kBandGroups && s_grp[threadIdx.x]) {
+      atomicAdd(&band[kBandBins + threadIdx.x], s_grp[threadIdx.x]);
+      s_grp[threadIdx.x] = 0;
+    }
+    if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+
+    if (threadIdx.x < kGateCtrN) s_at[threadIdx.x] = *(volatile unsigned long long*)&ctr[threadIdx.x];  // once per CTA: every warp's loads of one line would queue
+    __syncthreads();
+    unsigned long long extras = s_at[kGcExtra];
+    const unsigned long long lows = s_at[kGcLow], zeros = s_at[kGcZero], larger = s_at[kGcAbove];
+    const unsigned long long pushed = s_at[kGcPush], recs = s_at[kGcRec], drops = s_at[kGcDrop];
+    const unsigned long long merged = live + extras + lows, nz = merged - zeros;
+    auto grown = [&](unsigned long long e) { return nt_pass + (uint32_t)(e > n_free ? e - n_free : 0); };
+    nt = grown(extras);
+
+    // ------------------------------------------------------------ the cut
+    cut = SelState{};
+    if (a.n_keep > 0 && nz > (unsigned long long)a.n_keep) {
+      __syncthreads();  // sel's last readers are done
+      if (wid == 0) {
+        SelState t{};
+        t.mode = 1;
+        t.need = a.n_keep;
+        t.shift = 63;
+        t.kshift = 64;
+        if (banded && larger < (unsigned long long)a.n_keep) {
+          // largest first: the group of 128 bins, then the bin, that holds the need-th determinant
+          const unsigned need = (unsigned)((unsigned long long)a.n_keep - larger);
+          auto locate = [&](const unsigned* h, int n, unsigned want, int* where, unsigned* before, unsigned* count) {
+            // n / 32 consecutive bins per lane, from the last one down
+            const int per = n / 32;
+            unsigned v[4], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              v[q] = q < per ? __ldcg(&h[n - 1 - (lane * per + q)]) : 0u;
+              sum += v[q];
+            }
+            unsigned inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+              if (lane >= o) inc += x;
+            }
+            unsigned run = inc - sum;
+            int w_ = -1;
+            unsigned b_ = 0, c_ = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              if (q < per && w_ < 0 && run < want && run + v[q] >= want) {
+                w_ = n - 1 - (lane * per + q);
+                b_ = run;
+                c_ = v[q];
+              }
+              run += v[q];
+            }
+            const unsigned who = __ballot_sync(0xffffffffu, w_ >= 0);
+            if (!who) return false;
+            const int src = __ffs(who) - 1;
+            *where = __shfl_sync(0xffffffffu, w_, src);
+            *before = __shfl_sync(0xffffffffu, b_, src);
+            *count = __shfl_sync(0xffffffffu, c_, src);
+            return true;
+          };
+          int grp = 0, bin = 0;
+          unsigned before = 0, cnt = 0, b2 = 0;
+          if (locate(band + kBandBins, kBandGroups, need, &grp, &before, &cnt) &&
+              locate(band + grp * 128, 128, need - before, &bin, &b2, &cnt)) {
+            const unsigned rest = need - before - b2;  // of the bin's determinants, the largest `rest` are kept
+            bin += grp * 128;
+            if (rest == cnt) {
+              t.prefix = b_lo + ((unsigned long long)bin << kBandShift);
+              t.shift = kBandShift;
+              t.pass = 0x100 | 2;
+            } else if (cnt <= (unsigned)a.band_slots) {
+              BandEntry e{0, 0};
+              if (lane < (int)cnt) {
+                e.x = __ldcg(&slots[bin * a.band_slots + lane].x);
+                e.key = __ldcg(&slots[bin * a.band_slots + lane].key);
+              }
+              unsigned rank = 0;
+              for (unsigned q = 0; q < cnt; ++q) {
+                const unsigned long long x = __shfl_sync(0xffffffffu, e.x, q), k = __shfl_sync(0xffffffffu, e.key, q);
+                rank += x > e.x || (x == e.x && k < e.key);
+              }
+              const unsigned who = __ballot_sync(0xffffffffu, lane < (int)cnt && rank == rest - 1);
+              const int src = __ffs(who) - 1;
+              t.mode = 2;  // the cut is this determinant: exact |c| and bitstring
+              t.prefix = __shfl_sync(0xffffffffu, e.x, src);
+              t.kprefix = __shfl_sync(0xffffffffu, e.key, src);
+              t.shift = t.kshift = 0;
+              t.pass = 0x100 | 2;
+            }
+          }
+        }
+        if (lane == 0) sel = t;
+      }
+      __syncthreads();
+      if (!(sel.pass & 0x100)) {  // the general select, one pass and one barrier per digit
+        for (uint32_t i = gtid; i < kGateHistWords; i += gstride) a.hist[i] = 0;
+        if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+        bool decided = false;
+        for (int p = 0; p < kPasses && !decided; ++p) {
+          const bool keyphase = p >= kAbsPasses;
+          const int q = keyphase ? p - kAbsPasses : p;
+          const int lo = keyphase ? key_lo(q) : abs_lo(q), hi = keyphase ? key_hi(q) : abs_hi(q);
+          const unsigned dmask = (1u << (hi - lo)) - 1u;
+          unsigned* gh = a.hist + (size_t)p * kBins;
+          for (int t = threadIdx.x; t < kBins; t += blockDim.x) s_h0[t] = 0;
+          __syncthreads();
+          const unsigned long long pre = keyphase ? sel.kprefix : sel.prefix;
+          auto digit = [&](uint64_t k, double c) {
+            const uint64_t x = abs_bits(c);
+            if (x < a.min_abs_bits) return;
+            uint64_t v;
+            if (!keyphase) {
+              if (p > 0 && (x >> hi) != (pre >> hi)) return;
+              v = x;
+            } else {
+              if (x != sel.prefix) return;
+              if (hi < 64 && (k >> hi) != (pre >> hi)) return;
+              v = k;
+            }
+            atomicAdd(&s_h0[(v >> lo) & dmask], 1u);
+          };
+          for (uint32_t i = gtid; i < nt; i += gstride) {
+            const double c = __ldcg(&B[i]);
+            if (!dead(bits_of(c))) digit(keyphase ? __ldcg((const unsigned long long*)&a.keys[i]) : 0ull, c);
+          }
+          for (uint32_t i = gtid; i < (uint32_t)lows; i += gstride) digit(__ldcg((const unsigned long long*)&a.low_keys[i]), __ldcg(&a.low_amps[i]));
+          __syncthreads();
+          for (int t = threadIdx.x; t < kBins; t += blockDim.x)
+            if (s_h0[t]) atomicAdd(&gh[t], s_h0[t]);
+          if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+          for (int t = threadIdx.x; t < kBins; t += blockDim.x) s_h0[t] = __ldcg(&gh[t]);
+          if (threadIdx.x == 0) sel.bin = -1;
+          __syncthreads();
+          find_bin(s_h0, (int)dmask + 1, sel.need, !keyphase, sel, s_scan);
+          if (threadIdx.x == 0) {
+            int chosen = sel.bin;
+            if (chosen < 0) {  // cannot happen: total >= need
+              set_error(a.err, kDevBadState);
+              chosen = 0;
+            }
+            const long long need = sel.need - sel.cum, cnt = sel.cnt;
+            sel.need = need;
+            sel.pass = p + 1;
+            if (!keyphase) {
+              sel.prefix |= (unsigned long long)chosen << lo;
+              sel.shift = lo;
+              if (cnt == need) decided = true;
+              else if (lo == 0) sel.mode = 2;  // exact |c| ties at the cut
+            } else {
+              sel.kprefix |= (unsigned long long)chosen << lo;
+              sel.kshift = lo;
+              if (cnt == need || lo == 0) decided = true;
+            }
+            if (decided) sel.pass |= 0x100;
+          }
+          __syncthreads();
+          decided = (sel.pass & 0x100) != 0;
+        }
+      }
+      cut = sel;
+    }
+    // ------------------------------------------------------------ partners put aside that are kept after all
+    if (lows && (cut.mode == 0 || cut.prefix < filter)) {
+      for (uint32_t i0 = gtid - lane; i0 < (uint32_t)lows; i0 += gstride) {
+        const uint32_t i = i0 + lane;
+        uint64_t k = 0;
+        double c = 0.0;
+        bool want = false;
+        if (i < (uint32_t)lows) {
+          k = __ldcg((const unsigned long long*)&a.low_keys[i]);
+          c = __ldcg(&a.low_amps[i]);
+          want = keep_entry(cut, k, c, a.min_abs_bits);
+        }
+        const uint32_t p = want ? place(atomicAdd(&ctr[kGcExtra], 1ull), nt_pass) : kNoPos;
+        if (p != kNoPos) {
+          a.keys[p] = k;
+          B[p] = c;
+          if (p >= nt_pass) A[p] = __longlong_as_double((long long)kDead2);
+          if (!put_key(a.tab, a.tab_mask, mix64(k), p, ep)) set_error(a.err, kDevTableFull);
+          if (taped) {
+            const uint32_t r = __ldcg(&a.low_rec[i]);
+            const unsigned long long at = rec0 + (r & 0x7FFFFFFFu);
+            if (at < a.tape.cap) {
+              if (r >> 31) a.tape.pos[at].y = p;  // the new determinant is the upper one
+              else a.tape.pos[at].x = (a.tape.pos[at].x & 0x80000000u) | p;
+            }
+          }
+        }
+      }
+      if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+      if (threadIdx.x == 0) s_at[0] = *(volatile unsigned long long*)&ctr[kGcExtra];
+      __syncthreads();
+      extras = s_at[0];
+      nt = grown(extras);
+    }
+    if (gtid == 0 && a.stats) {
+      atomicAdd((unsigned long long*)&a.stats[0], 1ull);
+      atomicAdd((unsigned long long*)&a.stats[1], (unsigned long long)(cut.pass & 0xff));
+      atomicMax((unsigned long long*)&a.stats[6], merged);
+      atomicAdd((unsigned long long*)&a.stats[7], (unsigned long long)live);
+    }
+    head += extras < n_free ? extras : n_free;
+    tail += pushed;
+    used += extras;
+    rec0 += recs;
+    drop0 += drops;
+    live = cut.mode ? (uint64_t)a.n_keep : nz;
+    cur ^= 1;
+    const int d = dirty0;  // the next gate's set becomes the first
+    dirty0 = dirty1;
+    dirty1 = dirty2;
+    dirty2 = d;
+  }
+  // ---------------------------------------------------------------- the compact output and its index
+  if (taped && gtid == 0) {
+    a.tape.start[2 * a.n_ops] = rec0;
+    a.tape.start[2 * a.n_ops + 1] = drop0;
+    if (rec0 > a.tape.cap || drop0 > a.tape.drop_cap) set_error(a.err, kDevTableFull);  // cannot happen: sized for all
+  }
+  {
+    const double* A = a.amp[cur];
+    unsigned long long* kept = a.ctr + 3 * kGateCtrN;
+    for (uint32_t r0 = 0; r0 < nt; r0 += 32u * gstride) {
+      uint32_t mask = 0;
+      for (int it = 0; it < 32; ++it) {
+        const uint64_t i = (uint64_t)r0 + (uint64_t)it * gstride + gtid;
+        if (i >= nt) break;
+        const double c = __ldcg(&A[i]);
+        if (dead(bits_of(c))) continue;
+        if (keep_entry(cut, cut.mode == 2 ? __ldcg((const unsigned long long*)&a.keys[i]) : 0ull, c, a.min_abs_bits)) mask |= 1u << it;
+      }
+      unsigned inc = __popc(mask);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      if (lane == 31) s_scan[wid] = inc;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        long long run = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+          const long long v = s_scan[w];
+          s_scan[w] = run;
+          run += v;
+        }
+        s_base = run ? atomicAdd(kept, (unsigned long long)run) : 0ull;
+      }
+      __syncthreads();
+      unsigned long long pos = s_base + (unsigned long long)s_scan[wid] + (inc - __popc(mask));
+      __syncthreads();
+      for (; mask; mask &= mask - 1u, ++pos) {
+        const uint64_t i = (uint64_t)r0 + (uint64_t)(__ffs(mask) - 1) * gstride + gtid;
+        const uint64_t k = __ldcg((const unsigned long long*)&a.keys[i]);
+        a.out_keys[pos] = k;
+        a.out_amps[pos] = __ldcg(&A[i]);
+        if (a.out_pos) a.out_pos[pos] = (uint32_t)i;
+        if (!idx_insert(a.plain, a.plain_mask, k, pos)) set_error(a.err, kDevTableFull);
+      }
+    }
+  }
+  if (a.probe_ctr && (n_lookups | n_slots)) {
+    atomicAdd(&a.probe_ctr[0], (unsigned long long)n_lookups);
+    atomicAdd(&a.probe_ctr[1], (unsigned long long)n_slots);
+  }
+  if (gtid == 0) *a.n_state = (long long)live;
+  if (CLUSTER && nb > 1) cg::this_cluster().sync();  // the first CTA's counters are read until here
+}
+
+// ---------------------------------------------------------------- backward over the tape
+__global__ void nu_final_kernel(const double* amps, const double* sigma, const uint32_t* out_pos, const long long* n_ptr,
+                                const double* acc, double* nu, unsigned long long* zeros) {
+  const long long n = *n_ptr;
+  const double e = acc[0] / acc[1];
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double c = amps[i];
+    nu[out_pos[i]] = sigma[i] - e * c;
+    if (abs_bits(c) == 0) atomicAdd(zeros, 1ull);
+  }
+}
+
+__global__ void nu_realign_kernel(const uint64_t* keys, const uint32_t* out_pos, const long long* n_ptr, const IdxSlot* tab,
+                                  uint64_t mask, const double* nu_ck, double* nu) {
+  const long long n = *n_ptr;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int64_t j = idx_lookup(tab, mask, keys[i]);
+    nu[out_pos[i]] = j >= 0 ? nu_ck[j] : 0.0;
+  }
+}
+
+// Per gate, last first: every recorded block {L, U} (x before the gate, v = nu after it, c = cos, sn = sin)
+//   dE/dtheta += v_L (-sn x_L - s c x_U) + v_U (s c x_L - sn x_U),  v_L' = c v_L + s sn v_U,  v_U' = -s sn v_L + c v_U,
+// while nu of the determinants that the truncation before this gate dropped becomes 0 (their positions are in no
+// block of this gate).  One barrier per gate; everything else of nu stays where it is.
+template <bool CLUSTER>
+__global__ void __launch_bounds__(kGateThreads) back_kernel(BackArgs a) {
+  __shared__ double red[32];
+  __shared__ unsigned long long s_start[2][2];
+  const unsigned nb = gridDim.x;
+  unsigned round = 0;
+  const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, gstride = nb * blockDim.x;
+  // a gate's ranges are read once per CTA, its first blocks before the barrier of the gate after it
+  if (threadIdx.x < 4) s_start[threadIdx.x >> 1][threadIdx.x & 1] = a.tape.start[2 * (a.n_ops - 1) + threadIdx.x];
+  __syncthreads();
+  unsigned long long r0 = s_start[0][0], r1 = s_start[1][0], d0 = s_start[0][1], d1 = s_start[1][1];
+  uint2 p = make_uint2(0, 0);
+  double2 x = make_double2(0.0, 0.0);
+  if (r0 + gtid < r1) {
+    p = __ldcs(&a.tape.pos[r0 + gtid]);
+    x = __ldcs(&a.tape.x[r0 + gtid]);
+  }
+  for (int g = a.n_ops - 1; g >= 0; --g) {
+    const double c = a.cs[2 * g], sn = a.cs[2 * g + 1];
+    double acc = 0.0;
+    for (unsigned long long r = r0 + gtid; r < r1; r += gstride) {
+      if (r != r0 + gtid) {
+        p = __ldcs(&a.tape.pos[r]);
+        x = __ldcs(&a.tape.x[r]);
+      }
+      const double s = (p.x >> 31) ? -1.0 : 1.0;
+      const uint32_t L = p.x & 0x7FFFFFFFu, U = p.y;
+      const bool hl = L != (kNoPos & 0x7FFFFFFFu), hu = U != kNoPos;
+      const double vl = hl ? __ldcg(&a.nu[L]) : 0.0, vu = hu ? __ldcg(&a.nu[U]) : 0.0;
+      acc += vl * (-sn * x.x - s * c * x.y) + vu * (s * c * x.x - sn * x.y);
+      if (hl) a.nu[L] = c * vl + s * sn * vu;
+      if (hu) a.nu[U] = -s * sn * vl + c * vu;
+    }
+    for (unsigned long long r = d0 + gtid; r < d1; r += gstride) a.nu[__ldcs(&a.tape.drop[r])] = 0.0;
+    r1 = r0;
+    d1 = d0;
+    if (g > 0) {
+      if (threadIdx.x < 2) s_start[0][threadIdx.x] = a.tape.start[2 * (g - 1) + threadIdx.x];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      double t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (threadIdx.x == 0 && t != 0.0) atomicAdd(&a.dtheta[g], t);
+    }
+    if (g > 0) {
+      r0 = s_start[0][0];
+      d0 = s_start[0][1];
+      if (r0 + gtid < r1) {
+        p = __ldcs(&a.tape.pos[r0 + gtid]);
+        x = __ldcs(&a.tape.x[r0 + gtid]);
+      }
+      if (!gate_sync<CLUSTER>(a.bar, nb, round, a.err, a.timeout_ns)) return;
+    }
+  }
+}
+
+template <class K, class Args>
+cudaError_t launch_coop(K* kernel, const Args& a, int nblocks, bool clustered, size_t smem, cudaStream_t st) {
+  const cudaError_t e0 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e0 != cudaSuccess) return e0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(nblocks);
+  cfg.blockDim = dim3(kGateThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  if (clustered) {
+    if (nblocks > 8) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nblocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+template <class K>
+int cluster_fits(K* kernel, int ctas, size_t smem) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kGateThreads);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+}  // namespace
+
+int gate_cluster_fits(int ctas) {
+  const int f = cluster_fits(gates_kernel<true>, ctas, kGateSmem), b = cluster_fits(back_kernel<true>, ctas, 0);
+  return f < b ? f : b;
+}
+
+int gate_blocks_per_sm() {
+  int nb = 0;
+  if (cudaFuncSetAttribute(gates_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGateSmem) != cudaSuccess)
+    return 0;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, gates_kernel<false>, kGateThreads, kGateSmem) == cudaSuccess ? nb : 0;
+}
+
+int back_blocks_per_sm() {
+  int nb = 0;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, back_kernel<false>, kGateThreads, 0) == cudaSuccess ? nb : 0;
+}
+
+cudaError_t launch_gates(const GateArgs& a, int nblocks, bool clustered, cudaStream_t st) {
+  return clustered ? launch_coop(gates_kernel<true>, a, nblocks, true, kGateSmem, st)
+                   : launch_coop(gates_kernel<false>, a, nblocks, false, kGateSmem, st);
+}
+
+cudaError_t launch_back(const BackArgs& a, int nblocks, bool clustered, cudaStream_t st) {
+  return clustered ? launch_coop(back_kernel<true>, a, nblocks, true, 0, st)
+                   : launch_coop(back_kernel<false>, a, nblocks, false, 0, st);
+}
+
+cudaError_t launch_nu_final(const double* amps, const double* sigma, const uint32_t* out_pos, const long long* n,
+                            const double* acc, double* nu, unsigned long long* zeros, cudaStream_t st) {
+  nu_final_kernel<<<608, 256, 0, st>>>(amps, sigma, out_pos, n, acc, nu, zeros);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_nu_realign(const uint64_t* keys, const uint32_t* out_pos, const long long* n, const IdxSlot* tab,
+                              uint64_t mask, const double* nu_ck, double* nu, cudaStream_t st) {
+  nu_realign_kernel<<<608, 256, 0, st>>>(keys, out_pos, n, tab, mask, nu_ck, nu);
+  return cudaGetLastError();
+}
+
+}  // namespace swcs

@@ -39,11 +39,6 @@ struct AnsatzArgs {
   GridBar* bar;
   int* err;
   uint64_t timeout_ns;
-  // optional per-gate snapshots of the kept state (adjoint replay)
-  uint64_t* snap_keys;
-  double* snap_amps;
-  long long* snap_n;
-  int64_t snap_stride;
   long long* stats;  // optional: [0] gates, [1] select passes, [6] max |Phi|, [7] sum of input sizes
   int skip_arrive_block;  // test hook: this CTA never arrives at its first grid barrier (-1: off)
   unsigned long long* probe_ctr;  // optional (nullptr: off): [0] partner lookups, [1] slots they visited
@@ -264,23 +259,6 @@ cudaError_t launch_rbeta(const uint64_t* gkey, const long long* n, const uint32_
 
 // Adjoint (swcs_adjoint.cu).
 cudaError_t launch_build_index(const uint64_t* keys, const long long* n, IdxSlot* tab, uint64_t mask, cudaStream_t st);
-cudaError_t launch_nu_init(const double* amps, const double* sigma, const long long* n, const double* acc, double* nu,
-                           cudaStream_t st);
-struct AdjArgs {
-  const uint8_t* op;     // this gate
-  const double* cs;      // its (cos, sin)
-  const uint64_t* keys;  // S_g (before the gate), with its index table
-  const double* amps;
-  const long long* n;
-  const IdxSlot* tab;
-  uint64_t mask;
-  const IdxSlot* tab_nu;  // index of the arrays nu_in is aligned with (S_{g+1})
-  uint64_t mask_nu;
-  const double* nu_in;
-  double* nu_out;         // aligned with S_g
-  double* dtheta;         // accumulates the (unscaled) gradient of this gate
-};
-cudaError_t launch_adjoint_gate(const AdjArgs& a, int nblocks, cudaStream_t st);
 cudaError_t launch_scale_dtheta(double* d, int n, const double* acc, cudaStream_t st);
 
 // Screening network (swcs_mlp.cu).
