@@ -79,6 +79,7 @@ struct swcs_ctx {
 
   // in-place gate sequence: second amplitude array, partners put aside, free positions, positions of the output
   DevBuf amps_c, low_keys, low_amps, low_rec, ring, out_pos, band, band_slots;
+  DevBuf sort_k1, sort_v1, sort_k2, sort_v2, sort_cnt;  // copy-out in bitstring order
   int64_t max_state = 0;    // determinants the state buffers are sized for
   int cluster_ok[17] = {};  // clusters of k gate CTAs: 0 unknown, 1 fit, -1 do not
   // adjoint: checkpoints, tape of a segment, sigma, nu by position, nu and index of a checkpoint, gradient
@@ -93,6 +94,7 @@ struct swcs_ctx {
   // pairs of determinants (swcs_pairs.cu): string tables, grouped records, items; density matrices and the
   // contraction's integrals and work arrays (swcs_rdm.cu)
   DevBuf pr_tab, pr_slot, pr_pos, pr_rec, pr_oth, pr_idx, pr_items, rdm_tab, rdm_work, rdm_gamma;
+  bool rdm_tables_ready = false;  // rdm_tab holds the loaded Hamiltonian's integrals
   int opt_pairs = -1;  // pool sweep from density matrices: -1 automatic, 0 never, 1 wherever it applies
 
   // external sigma table
@@ -854,7 +856,7 @@ int energy_rows(swcs_ctx* c, double* sig_out) {
 //             states crowd around the reference).
 bool use_density_matrices(swcs_ctx* c, int64_t nd) {
   if (c->opt_sweep != 0 || c->opt_count_probes || c->opt_pairs == 0) return false;
-  if (c->no < 2 || nd > kMaxPairDets || !c->rdm_tab.p) return false;
+  if (c->no < 2 || nd > kMaxPairDets) return false;
   if (c->opt_pairs == 1) return true;
   if (c->NB <= 0 || c->NB > (1 << 22)) return true;  // no row sweep there: the hashed table is slower than either
   const double n = (double)nd, m = c->n / 2, no = c->no, nv = c->nv;
@@ -872,7 +874,15 @@ bool use_density_matrices(swcs_ctx* c, int64_t nd) {
 int sweep_density(swcs_ctx* c, double* d_g, int64_t nd) {
   const int m = c->n / 2;
   const size_t gd = rdm_gamma_doubles(m);
-  if (ensure(c, c->rdm_gamma, gd * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8)) return 1;
+  if (ensure(c, c->rdm_gamma, gd * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8) ||
+      ensure(c, c->rdm_tab, rdm_table_doubles(m) * 8))
+    return 1;
+  if (!c->rdm_tables_ready) {  // once per Hamiltonian, from its staged copy
+    CK(launch_k(c, kKOther, [&] {
+      return launch_rdm_tables((const double*)c->gstage.p, c->n, rdm_tables((double*)c->rdm_tab.p, m), c->st);
+    }));
+    c->rdm_tables_ready = true;
+  }
   RdmArgs a{};
   const int r = pair_args(c, nd, false, &a.P);
   if (r) return r;
@@ -1038,7 +1048,7 @@ int swcs_destroy(swcs_ctx* c) {
                     &c->rbeta, &c->gab, &c->kab, &c->gorig,
                     &c->ck_keys, &c->ck_amps, &c->ck_n, &c->tp_pos, &c->tp_x, &c->tp_drop, &c->tp_start, &c->sigma,
                     &c->nu0, &c->nu1, &c->atab0, &c->dth, &c->amps_c, &c->low_keys, &c->low_amps, &c->low_rec, &c->ring,
-                    &c->out_pos, &c->band, &c->band_slots, &c->pool_dev, &c->selbits, &c->feat,
+                    &c->out_pos, &c->band, &c->band_slots, &c->sort_k1, &c->sort_v1, &c->sort_k2, &c->sort_v2, &c->sort_cnt, &c->pool_dev, &c->selbits, &c->feat,
                     &c->ypred, &c->topk_hist, &c->topk_ctl, &c->occ, &c->prb, &c->ab_cnt, &c->ab_list,
                     &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items,
                     &c->rdm_tab, &c->rdm_work, &c->rdm_gamma};
@@ -1077,14 +1087,7 @@ int swcs_load_hamiltonian(swcs_ctx* c, const double* h_h, const double* h_g, int
   CK(cudaMemcpyAsync(c->h.p, h_h, n2 * 8, cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(c->gstage.p, h_g, n4 * 8, cudaMemcpyHostToDevice, c->st));
   CK(launch_k(c, kKOther, [&] { return launch_pack_hamiltonian((const double*)c->gstage.p, n, (double*)c->J.p, (double*)c->Ws.p, (double*)c->G.p, c->st); }));
-  if (c->no >= 2) {  // the density-matrix contraction's layout of the same integrals
-    if ((r = ensure(c, c->rdm_tab, rdm_table_doubles(n / 2) * 8))) return r;
-    CK(launch_k(c, kKOther, [&] {
-      return launch_rdm_tables((const double*)c->gstage.p, n, rdm_tables((double*)c->rdm_tab.p, n / 2), c->st);
-    }));
-  } else {
-    release(c->rdm_tab);
-  }
+  c->rdm_tables_ready = false;
   std::vector<int> opd, ops1;
   build_pool(c, opd, ops1);
   {
@@ -1470,6 +1473,25 @@ int swcs_state_size(swcs_ctx* c, int64_t* n_out) {
   return SWCS_OK;
 }
 
+// The state's determinants with their values (state order) to the host, sorted by bitstring.
+static int copy_out_sorted(swcs_ctx* c, const double* vals, int64_t n, uint64_t* h_keys, double* h_vals, const char* where) {
+  int r;
+  DevBuf* kb[2] = {&c->sort_k1, &c->sort_k2};
+  DevBuf* vb[2] = {&c->sort_v1, &c->sort_v2};
+  for (int i = 0; i < 2; ++i)
+    if ((r = ensure(c, *kb[i], (size_t)n * 8)) || (r = ensure(c, *vb[i], (size_t)n * 8))) return r;
+  if ((r = ensure(c, c->sort_cnt, sort_count_words(n) * 4))) return r;
+  bool second = false;
+  CK(launch_k(c, kKOther, [&] {
+    return launch_sort_pairs((const uint64_t*)c->keys_a.p, vals, (uint64_t*)kb[0]->p, (double*)vb[0]->p, (uint64_t*)kb[1]->p,
+                             (double*)vb[1]->p, n, c->n, (uint32_t*)c->sort_cnt.p, &second, c->st);
+  }));
+  c->launches += 3 * ((c->n + 7) / 8) - 1;
+  CK(cudaMemcpyAsync(h_keys, kb[second]->p, 8 * n, cudaMemcpyDeviceToHost, c->st));
+  CK(cudaMemcpyAsync(h_vals, vb[second]->p, 8 * n, cudaMemcpyDeviceToHost, c->st));
+  return check_device(c, where);
+}
+
 int swcs_get_state(swcs_ctx* c, uint64_t* keys, double* amps, int64_t cap, int64_t* n_out) {
   int r = need_state(c);
   if (r) return r;
@@ -1478,18 +1500,7 @@ int swcs_get_state(swcs_ctx* c, uint64_t* keys, double* amps, int64_t cap, int64
   if (n < 0) return fail(c, SWCS_ERR_CUDA, "cannot read state size");
   if (n_out) *n_out = n;
   if (cap < n || n == 0) return SWCS_OK;
-  std::vector<uint64_t> k(n);
-  std::vector<double> a(n);
-  CK(cudaMemcpy(k.data(), c->keys_a.p, 8 * n, cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(a.data(), c->amps_a.p, 8 * n, cudaMemcpyDeviceToHost));
-  std::vector<int64_t> ord(n);
-  for (int64_t i = 0; i < n; ++i) ord[i] = i;
-  std::sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return k[x] < k[y]; });
-  for (int64_t i = 0; i < n; ++i) {
-    keys[i] = k[ord[i]];
-    amps[i] = a[ord[i]];
-  }
-  return SWCS_OK;
+  return copy_out_sorted(c, (const double*)c->amps_a.p, n, keys, amps, "swcs_get_state");
 }
 
 int swcs_set_state(swcs_ctx* c, const uint64_t* keys, const double* amps, int64_t n) {
@@ -1585,19 +1596,7 @@ int swcs_get_sigma(swcs_ctx* c, uint64_t* keys, double* sigma, int64_t cap, int6
   CK(launch_k(c, kKEnergy, [&] {
     return launch_energy_sigma(ham_dev(c), state_dev(c), k->acc, (double*)c->sigma.p, c->nsm * sigma_blocks_per_sm(), c->st);
   }));
-  std::vector<uint64_t> kk(n);
-  std::vector<double> ss(n);
-  CK(cudaMemcpyAsync(kk.data(), c->keys_a.p, 8 * n, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaMemcpyAsync(ss.data(), c->sigma.p, 8 * n, cudaMemcpyDeviceToHost, c->st));
-  if ((r = check_device(c, "swcs_get_sigma"))) return r;
-  std::vector<int64_t> ord(n);
-  for (int64_t i = 0; i < n; ++i) ord[i] = i;
-  std::sort(ord.begin(), ord.end(), [&](int64_t x, int64_t y) { return kk[x] < kk[y]; });
-  for (int64_t i = 0; i < n; ++i) {
-    keys[i] = kk[ord[i]];
-    sigma[i] = ss[ord[i]];
-  }
-  return SWCS_OK;
+  return copy_out_sorted(c, (const double*)c->sigma.p, n, keys, sigma, "swcs_get_sigma");
 }
 
 int swcs_sigma_at(swcs_ctx* c, const uint64_t* keys, int64_t n, double* sigma) {

@@ -338,6 +338,11 @@ cudaError_t launch_topk(const float* y, int64_t n, int64_t k, unsigned* hist, un
 cudaError_t launch_subset_bits(const int64_t* subset, int64_t n, uint32_t* bits, int64_t n_pool, cudaStream_t st);
 cudaError_t launch_log_abs(const double* g, int64_t n, float* t, cudaStream_t st);
 
+// Copy-out order (swcs_sort.cu).
+size_t sort_count_words(int64_t n);
+cudaError_t launch_sort_pairs(const uint64_t* k0, const double* v0, uint64_t* k1, double* v1, uint64_t* k2, double* v2,
+                              int64_t n, int bits, uint32_t* counts, bool* in_k2, cudaStream_t st);
+
 // Hamiltonian preparation from the full <pq||rs> array on the device.
 cudaError_t launch_pack_hamiltonian(const double* g_full, int n, double* J, double* Ws, double* G,
                                     cudaStream_t st);

@@ -57,7 +57,7 @@ struct PairArgs {
 cudaError_t launch_pairs_energy(const PairArgs& a, int64_t n, int nsm, cudaStream_t st);
 cudaError_t launch_pairs_gamma(const PairArgs& a, int64_t n, int nsm, cudaStream_t st);
 
-// Tables of the Hamiltonian for the contraction, laid out once when it is loaded (m spatial orbitals, P = m(m-1)/2):
+// Tables of the Hamiltonian for the contraction, laid out once per Hamiltonian (m spatial orbitals, P = m(m-1)/2):
 //   vss [2][m][P][m]     g(p s, x s; y s, z s), pair (y < z), at ((s m + x) P + pair) m + p
 //   vos [2][m][m][m][m]  g(p s, x o; y o, z s), o = 1 - s, at (((s m + x) m + y) m + z) m + p
 //   v2s [2][P][P]        g(p s, q s; y s, z s)
