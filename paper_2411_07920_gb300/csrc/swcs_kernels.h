@@ -262,7 +262,7 @@ cudaError_t launch_build_index(const uint64_t* keys, const long long* n, IdxSlot
 cudaError_t launch_scale_dtheta(double* d, int n, const double* acc, cudaStream_t st);
 
 // Screening network (swcs_mlp.cu).
-enum GemmMode { kGemmF32 = 0, kGemmReluBf16 = 1, kGemmReluBf16Dot = 2 };
+enum GemmMode { kGemmF32 = 0, kGemmReluBf16 = 1, kGemmReluBf16Dot = 2, kGemmMaskBf16 = 3 };
 struct GemmArgs {
   const __nv_bfloat16* A;  // [M x K], row stride lda (elements), K contiguous
   const __nv_bfloat16* B;  // [N x K], row stride ldb
@@ -277,6 +277,18 @@ struct GemmArgs {
   float b3;
   float* y;
   int* err;
+  // what the pipelined kernel's epilogue also does in training (nullptr: not wanted)
+  __nv_bfloat16* out_t;       // [N x ldt] the BF16 result transposed (kGemmMaskBf16: only this), rows M .. ldt zero
+  int ldt;
+  const __nv_bfloat16* mask;  // kGemmMaskBf16: [M x ldo], the result is bf16(C) where mask > 0, else 0
+  float* colsum;              // [N] += column sums of the BF16 result (kGemmMaskBf16) or of dz (Dot with target)
+  const float* target;        // kGemmReluBf16Dot: [M] targets of the mean squared error over M rows; then
+  const float* b3_dev;        //   y gets b3_dev[0] added, dy = 2 (y - target) / M,
+  double* loss;               //   loss += the error,
+  __nv_bfloat16* dz;          //   dz [M x ldo] = bf16(dy w3 (out > 0)), and dz_t its transpose [N x ldt],
+  __nv_bfloat16* dz_t;
+  float* dw3;                 //   dw3 [N] += dy out, db3 += dy
+  float* db3;
 };
 struct MlpParams {
   float* master;

@@ -230,15 +230,79 @@ __device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* map, int x,
       : "memory");
 }
 
+// 16 consecutive parameters, the same for every lane, in 16-byte loads.
+__device__ __forceinline__ void params16(const float* p, float* v) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p) + i);
+    v[4 * i] = q.x;
+    v[4 * i + 1] = q.y;
+    v[4 * i + 2] = q.z;
+    v[4 * i + 3] = q.w;
+  }
+}
+__device__ __forceinline__ void params16(const __nv_bfloat16* p, float* v) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p) + i);
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[8 * i + 2 * k] = __uint_as_float(w[k] << 16);
+      v[8 * i + 2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+    }
+  }
+}
+
+// 16 BF16 values of one row, contiguous (32 bytes).
+__device__ __forceinline__ void store_row16(__nv_bfloat16* p, const __nv_bfloat16* h) {
+  uint32_t w[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    w[i] = (uint32_t)__bfloat16_as_ushort(h[2 * i]) | ((uint32_t)__bfloat16_as_ushort(h[2 * i + 1]) << 16);
+  reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+  reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+// The same values down 16 columns of the transpose: a warp's rows are consecutive, so each store is 64 bytes.
+__device__ __forceinline__ void store_col16(__nv_bfloat16* p, int ld, const __nv_bfloat16* h) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) p[(size_t)i * ld] = h[i];
+}
+
+// Sums of 16 values over the warp's lanes, added to acc[0..15]: halves exchanged and added until each lane holds one
+// column (16 shuffles instead of 80).
+__device__ __forceinline__ void add_columns16(float* v, float* acc, int lane) {
+#pragma unroll
+  for (int w = 8; w >= 1; w >>= 1) {
+    const bool up = lane & (2 * w);
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const float give = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * w);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  if (!(lane & 1)) atomicAdd(&acc[(lane >> 4 & 1) * 8 + (lane >> 3 & 1) * 4 + (lane >> 2 & 1) * 2 + (lane >> 1 & 1)], v[0]);
+}
+
+constexpr int kTmaThreads = 128 * kDotGroups;  // four warps (one per tensor-memory lane quadrant) for each column group
+
 // C = A B^T for one 128-row tile and K-chunks [c0, c1) of kc elements (this CTA's split of K).  Stage s
 // holds A as kc/8 column blocks of 128 rows x 16 B (one TMA box each: LBO 2 KB, SBO 128 B) and B as kc/8
 // blocks of N x 16 B (LBO N x 16 B, SBO 128 B).
-__global__ void __launch_bounds__(kGemmThreads)
+//
+// At training sizes (64 row tiles, K at most 256) the epilogue is the kernel: 16 warps share it by row quadrant and
+// column group, parameters and row-major results move in 16-byte accesses, and what used to be kernels of their own
+// between the GEMMs -- the loss and its gradient, the masks, the transposes, the column sums -- happens while the
+// values are in registers.  The gradient of 8,192 rows: 279 us with 128-thread epilogues and 12 further launches.
+__global__ void __launch_bounds__(kTmaThreads)
 mlp_gemm_tma_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, GemmArgs g,
                     int kc, int splits) {
   extern __shared__ __align__(128) uint8_t dsm[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], fin;
   __shared__ uint32_t tmem_holder;
+  __shared__ float sPart[kDotGroups][128], sDy[128], sSum[2][256];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * 128;
   const int ncols = g.N <= 32 ? 32 : (g.N <= 64 ? 64 : (g.N <= 128 ? 128 : 256));
@@ -262,6 +326,7 @@ mlp_gemm_tma_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     mbar_init1(&fin);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < 512; i += kTmaThreads) (&sSum[0][0])[i] = 0.f;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -315,47 +380,124 @@ mlp_gemm_tma_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   if (!mbar_wait(smem_u32(&fin), 0)) bad = true;
   bad = __syncthreads_or(bad) != 0;  // one decision for the whole CTA before the warp-wide tensor-memory loads
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // ---------------- epilogue: thread t owns row m0 + t (TMEM lane t)
-  const int row = m0 + threadIdx.x;
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;  // dot-product partial sums (kDotGroups)
-  const bool empty_split = c0 >= c1;               // no chunk: nothing was accumulated
-  if (!bad && !empty_split) {
-    for (int cc = 0; cc < g.N; cc += 16) {
+  // ---------------- epilogue: the warp's lanes are 32 rows, its group's columns [cb, ce)
+  const int q = warp & 3, grp = warp >> 2, r = q * 32 + lane, row = m0 + r;
+  const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+  const int cb = dot_group_begin(grp, g.N / 16) * 16, ce = dot_group_begin(grp + 1, g.N / 16) * 16;
+  const bool in = row < g.M, in_t = row < g.ldt;
+  const bool dot = g.mode == kGemmReluBf16Dot;
+  float part = 0.f;  // this group's part of the dot product
+  if (!bad && c0 < c1) {  // (no chunk: nothing was accumulated)
+    for (int cc = cb; cc < ce; cc += 16) {
       float v[16];
       tmem_ld16(tmem + lane_base + (uint32_t)cc, v);
-      int grp = 0;
-      while (grp < kDotGroups - 1 && dot_group_begin(grp + 1, g.N / 16) <= cc / 16) ++grp;
-      float part = grp == 0 ? p0 : (grp == 1 ? p1 : (grp == 2 ? p2 : p3));
-      if (row < g.M) {
-        if (g.mode == kGemmF32) {
+      if (g.mode == kGemmF32) {
+        if (in) {
           float* o = g.out_f32 + (size_t)row * g.ldo + cc;
-          if (splits > 1) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) atomicAdd(&o[i], v[i]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) o[i] = v[i];
-          }
-        } else {
-          __nv_bfloat16* o = g.out_bf16 + (size_t)row * g.ldo + cc;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float z = v[i] + (g.bias ? g.bias[cc + i] : 0.f);
-            z = z > 0.f ? z : 0.f;
-            const __nv_bfloat16 hb = __float2bfloat16_rn(z);
-            o[i] = hb;
-            if (g.mode == kGemmReluBf16Dot) part += __bfloat162float(hb) * __bfloat162float(g.w3[cc + i]);
+          for (int i = 0; i < 16; i += 4) {
+            const float4 f4 = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            if (splits > 1) atomicAdd(reinterpret_cast<float4*>(o + i), f4);
+            else *reinterpret_cast<float4*>(o + i) = f4;
           }
         }
+        __syncwarp();
+        continue;
       }
-      if (grp == 0) p0 = part;
-      else if (grp == 1) p1 = part;
-      else if (grp == 2) p2 = part;
-      else p3 = part;
+      __nv_bfloat16 h[16];
+      if (g.mode == kGemmMaskBf16) {
+        float mk[16];
+        if (in) params16(g.mask + (size_t)row * g.ldo + cc, mk);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h[i] = __float2bfloat16_rn(in && mk[i] > 0.f ? v[i] : 0.f);
+        if (in_t) store_col16(g.out_t + (size_t)cc * g.ldt + row, g.ldt, h);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __bfloat162float(h[i]);
+        add_columns16(v, &sSum[0][cc], lane);
+        continue;
+      }
+      float b[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) b[i] = 0.f;
+      if (g.bias) params16(g.bias + cc, b);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        float z = v[i] + b[i];
+        z = z > 0.f ? z : 0.f;
+        h[i] = __float2bfloat16_rn(in ? z : 0.f);
+      }
+      if (in) store_row16(g.out_bf16 + (size_t)row * g.ldo + cc, h);
+      if (g.out_t && in_t) store_col16(g.out_t + (size_t)cc * g.ldt + row, g.ldt, h);
+      if (dot) {
+        float w3[16];
+        params16(g.w3 + cc, w3);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part += __bfloat162float(h[i]) * w3[i];
+      }
     }
   }
-  if (g.mode == kGemmReluBf16Dot && row < g.M && !bad) g.y[row] = (((p0 + p1) + p2) + p3) + g.b3;
+  if (dot) {
+    sPart[grp][r] = part;
+    __syncthreads();
+    if (grp == 0) {
+      float y = (((sPart[0][r] + sPart[1][r]) + sPart[2][r]) + sPart[3][r]) + g.b3;
+      float dy = 0.f;
+      double err2 = 0.0;
+      if (g.target) {
+        if (in && !bad) {
+          y += __ldg(g.b3_dev);
+          const float d = y - __ldg(&g.target[row]);
+          dy = 2.f * d / (float)g.M;
+          err2 = (double)d * d;
+        }
+        sDy[r] = dy;
+        float sdy = dy;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          err2 += __shfl_xor_sync(0xffffffffu, err2, o);
+          sdy += __shfl_xor_sync(0xffffffffu, sdy, o);
+        }
+        if (lane == 0) {
+          if (err2 != 0.0) atomicAdd(g.loss, err2 / g.M);
+          atomicAdd(g.db3, sdy);
+        }
+      }
+      if (in && !bad) g.y[row] = y;
+    }
+    if (g.target) {
+      __syncthreads();
+      const float dy = sDy[r];
+      if (!bad) {
+        for (int cc = cb; cc < ce; cc += 16) {  // dz = bf16(dy w3 (h > 0)), h formed again from the accumulator
+          float v[16], b[16], w3[16], s1[16];
+          __nv_bfloat16 h[16];
+          tmem_ld16(tmem + lane_base + (uint32_t)cc, v);
+          params16(g.bias + cc, b);
+          params16(g.w3 + cc, w3);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            float z = v[i] + b[i];
+            z = z > 0.f ? z : 0.f;
+            const float hf = __bfloat162float(__float2bfloat16_rn(z));
+            h[i] = __float2bfloat16_rn(in && hf > 0.f ? dy * w3[i] : 0.f);
+            s1[i] = in ? dy * hf : 0.f;
+            v[i] = __bfloat162float(h[i]);
+          }
+          if (in) store_row16(g.dz + (size_t)row * g.ldo + cc, h);
+          if (in_t) store_col16(g.dz_t + (size_t)cc * g.ldt + row, g.ldt, h);
+          add_columns16(v, &sSum[0][cc], lane);
+          add_columns16(s1, &sSum[1][cc], lane);
+        }
+      }
+    }
+  }
+  if (g.colsum) {
+    __syncthreads();
+    for (int j = threadIdx.x; j < g.N; j += kTmaThreads) {
+      if (sSum[0][j] != 0.f) atomicAdd(&g.colsum[j], sSum[0][j]);
+      if (g.dw3 && sSum[1][j] != 0.f) atomicAdd(&g.dw3[j], sSum[1][j]);
+    }
+  }
   if (bad && g.err) set_error(g.err, kDevTimeout);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -488,7 +630,7 @@ cudaError_t launch_mlp_gemm_tma(const CUtensorMap& tm_a, const CUtensorMap& tm_b
     if (e != cudaSuccess) return e;
     attr = smem;
   }
-  mlp_gemm_tma_kernel<<<dim3((g.M + 127) / 128, splits), kGemmThreads, smem, st>>>(tm_a, tm_b, g, kc, splits);
+  mlp_gemm_tma_kernel<<<dim3((g.M + 127) / 128, splits), kTmaThreads, smem, st>>>(tm_a, tm_b, g, kc, splits);
   return cudaGetLastError();
 }
 

@@ -90,6 +90,7 @@ GemmArgs gemm(swcs_mlp* m, const __nv_bfloat16* A, int lda, const __nv_bfloat16*
 }
 
 bool k_major_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows);
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 // C = A B^T through the pipelined kernel when both operands have tensor maps (K contiguous, 16-byte aligned),
 // else through the staged one.  may_split: the FP32 output holds zeros, so K may be split over CTAs.
@@ -106,6 +107,8 @@ int run_gemm(swcs_mlp* m, const GemmArgs& g, bool may_split) {
       splits = std::max(1, std::min(nch / 4, (2 * nsm) / tiles));  // at least four K-chunks per CTA
     }
     MCK(launch_mlp_gemm_tma(ta, tb, g, splits, m->st));
+  } else if (g.out_t || g.target || g.mode == kGemmMaskBf16) {
+    return mfail(m, SWCS_ERR_CUDA, "mlp: no tensor map for a training GEMM");
   } else {
     MCK(launch_mlp_gemm(g, m->st));
   }
@@ -205,6 +208,50 @@ int add_b3(swcs_mlp* m, float* y, int64_t n) {
   return SWCS_OK;
 }
 
+// Whether every GEMM of a gradient of n rows runs pipelined, with its fused epilogue.
+bool fused_training(const swcs_mlp* m, const __nv_bfloat16* x) {
+  return m->pipeline && tensor_map_encoder() && !((uintptr_t)x & 15) && m->p.off_b1 % 4 == 0 && m->p.off_b2 % 4 == 0;
+}
+
+// Loss, activations and gradients with the elementwise work in the GEMMs' epilogues (mlp_gemm_tma_kernel).
+int grads_fused(swcs_mlp* m, const __nv_bfloat16* x, const float* t, int64_t n, int Bpad) {
+  const int W = m->p.width, D = m->p.d_in;
+  int r;
+  MCK(launch_mlp_transpose(x, (int)n, D, Bpad, m->Xt, m->st));
+  GemmArgs g1 = gemm(m, x, D, m->p.W1b, D, (int)n, W, D, kGemmReluBf16);
+  g1.bias = m->p.master + m->p.off_b1;
+  g1.out_bf16 = m->H1;
+  g1.ldo = W;
+  g1.out_t = m->H1t;
+  g1.ldt = Bpad;
+  if ((r = run_gemm(m, g1, false))) return r;
+  GemmArgs g2 = gemm(m, m->H1, W, m->p.W2b, W, (int)n, W, W, kGemmReluBf16Dot);
+  g2.bias = m->p.master + m->p.off_b2;
+  g2.out_bf16 = m->H2;
+  g2.ldo = W;
+  g2.w3 = m->p.w3b;
+  g2.y = m->y;
+  g2.target = t;
+  g2.b3_dev = m->p.master + m->p.off_b3;
+  g2.loss = m->loss;
+  g2.dz = m->dZ2;
+  g2.dz_t = m->dZ2t;
+  g2.ldt = Bpad;
+  g2.colsum = m->grad + m->p.off_b2;
+  g2.dw3 = m->grad + m->p.off_w3;
+  g2.db3 = m->grad + m->p.off_b3;
+  if ((r = run_gemm(m, g2, false))) return r;
+  GemmArgs g3 = gemm(m, m->dZ2, W, m->p.W2tb, W, (int)n, W, W, kGemmMaskBf16);  // dZ1 = (dZ2 W2) (H1 > 0)
+  g3.mask = m->H1;
+  g3.ldo = W;
+  g3.out_t = m->dZ1t;
+  g3.ldt = Bpad;
+  g3.colsum = m->grad + m->p.off_b1;
+  if ((r = run_gemm(m, g3, false))) return r;
+  m->launches += 4;
+  return SWCS_OK;
+}
+
 int grads(swcs_mlp* m, const __nv_bfloat16* x, const float* t, int64_t n, double* d_loss) {
   const int W = m->p.width, D = m->p.d_in;
   int r;
@@ -212,20 +259,25 @@ int grads(swcs_mlp* m, const __nv_bfloat16* x, const float* t, int64_t n, double
   const int Bpad = (int)(((n + 31) / 32) * 32);
   MCK(cudaMemsetAsync(m->grad, 0, sizeof(float) * m->p.n_params, m->st));
   MCK(cudaMemsetAsync(m->loss, 0, sizeof(double), m->st));
-  if ((r = forward(m, x, n, m->y)) || (r = add_b3(m, m->y, n))) return r;
-  MCK(launch_mlp_dy(m->y, t, (int)n, m->dy, m->loss, m->st));
-  MCK(launch_mlp_dz2(m->dy, m->p.w3b, m->H2, (int)n, W, m->dZ2, m->grad + m->p.off_w3, m->grad + m->p.off_b3, m->st));
-  GemmArgs g3 = gemm(m, m->dZ2, W, m->p.W2tb, W, (int)n, W, W, kGemmF32);  // dH1 = dZ2 W2
-  g3.out_f32 = m->dH1;
-  g3.ldo = W;
-  if ((r = run_gemm(m, g3, false))) return r;
-  MCK(launch_mlp_dz1(m->dH1, m->H1, (size_t)n * W, m->dZ1, m->st));
-  MCK(launch_mlp_colsum(m->dZ2, (int)n, W, m->grad + m->p.off_b2, m->st));
-  MCK(launch_mlp_colsum(m->dZ1, (int)n, W, m->grad + m->p.off_b1, m->st));
-  MCK(launch_mlp_transpose(m->dZ2, (int)n, W, Bpad, m->dZ2t, m->st));
-  MCK(launch_mlp_transpose(m->H1, (int)n, W, Bpad, m->H1t, m->st));
-  MCK(launch_mlp_transpose(m->dZ1, (int)n, W, Bpad, m->dZ1t, m->st));
-  MCK(launch_mlp_transpose(x, (int)n, D, Bpad, m->Xt, m->st));
+  if (fused_training(m, x)) {
+    if ((r = grads_fused(m, x, t, n, Bpad))) return r;
+  } else {
+    if ((r = forward(m, x, n, m->y)) || (r = add_b3(m, m->y, n))) return r;
+    MCK(launch_mlp_dy(m->y, t, (int)n, m->dy, m->loss, m->st));
+    MCK(launch_mlp_dz2(m->dy, m->p.w3b, m->H2, (int)n, W, m->dZ2, m->grad + m->p.off_w3, m->grad + m->p.off_b3, m->st));
+    GemmArgs g3 = gemm(m, m->dZ2, W, m->p.W2tb, W, (int)n, W, W, kGemmF32);  // dH1 = dZ2 W2
+    g3.out_f32 = m->dH1;
+    g3.ldo = W;
+    if ((r = run_gemm(m, g3, false))) return r;
+    MCK(launch_mlp_dz1(m->dH1, m->H1, (size_t)n * W, m->dZ1, m->st));
+    MCK(launch_mlp_colsum(m->dZ2, (int)n, W, m->grad + m->p.off_b2, m->st));
+    MCK(launch_mlp_colsum(m->dZ1, (int)n, W, m->grad + m->p.off_b1, m->st));
+    MCK(launch_mlp_transpose(m->dZ2, (int)n, W, Bpad, m->dZ2t, m->st));
+    MCK(launch_mlp_transpose(m->H1, (int)n, W, Bpad, m->H1t, m->st));
+    MCK(launch_mlp_transpose(m->dZ1, (int)n, W, Bpad, m->dZ1t, m->st));
+    MCK(launch_mlp_transpose(x, (int)n, D, Bpad, m->Xt, m->st));
+    m->launches += 10;
+  }
   GemmArgs g4 = gemm(m, m->dZ2t, Bpad, m->H1t, Bpad, W, W, Bpad, kGemmF32);  // dW2 = dZ2^T H1
   g4.out_f32 = m->grad + m->p.off_W2;
   g4.ldo = W;
@@ -234,7 +286,7 @@ int grads(swcs_mlp* m, const __nv_bfloat16* x, const float* t, int64_t n, double
   g5.out_f32 = m->grad + m->p.off_W1;
   g5.ldo = D;
   if ((r = run_gemm(m, g5, true))) return r;
-  m->launches += 12;
+  m->launches += 2;
   if (d_loss) MCK(cudaMemcpyAsync(d_loss, m->loss, sizeof(double), cudaMemcpyDeviceToDevice, m->st));
   return SWCS_OK;
 }
