@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -103,9 +104,10 @@ struct swcs_ctx {
   double ext_distinct_last = 0.0;
   int64_t stats[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 
-  // pinned host staging
+  // pinned host staging: the status head, then gates on their way to the device
   void* pin = nullptr;
   size_t pin_bytes = 0;
+  bool pin_busy = false;  // copies out of it may be in flight
 
   // per-kernel event timing (swcs_profile_*) and launch count
   bool prof = false;
@@ -122,24 +124,31 @@ struct swcs_ctx {
 
 namespace {
 
-// Layout of the small control block on the device.
-struct Ctrl {
+// What a synchronising call reads back of the control block, in one copy.
+struct Status {
   long long n_state;
   int tab_cur;
   int err;
+  double eout[2];
+  unsigned long long zeros;  // exactly zero amplitudes kept by the adjoint's projectors
+};
+
+// Layout of the small control block on the device.
+struct Ctrl : Status {
   GridBar bar;
   unsigned long long ctr[12];
   unsigned long long gate_ctr[3 * kGateCtrN + 1];  // in-place gate sequence
-  unsigned long long zeros;                        // exactly zero amplitudes kept by the adjoint's projectors
   long long stats[8];
-  double acc[2];
-  PairCtl pairs;  // right after acc: one memset clears both
-  double eout[2];
+  double acc[2];  // from here to row_next: cleared by one memset at the start of a sweep or an energy
+  PairCtl pairs;
   unsigned long long n_distinct;
+  unsigned row_next;  // the row sweep's next target
   double ovl[3];  // swcs_overlap: <state|given>, <given|given>, <state|state>
   unsigned long long probes[4];  // hash probes: gate lookups, their slots, row-sweep lookups, their slots
-  unsigned row_next;  // the row sweep's next target
 };
+constexpr size_t kSweepClear = offsetof(Ctrl, row_next) + sizeof(unsigned) - offsetof(Ctrl, acc);
+constexpr size_t kPinStatus = 64;  // head of the pinned staging buffer
+static_assert(sizeof(Status) <= kPinStatus, "status head");
 
 int fail(swcs_ctx* c, int code, const char* fmt, ...) {
   char buf[512];
@@ -184,6 +193,7 @@ void release(DevBuf& b) {
 
 int ensure_pinned(swcs_ctx* c, size_t bytes) {
   if (c->pin_bytes >= bytes) return SWCS_OK;
+  if (c->pin_busy) cudaStreamSynchronize(c->st);
   if (c->pin) cudaFreeHost(c->pin);
   c->pin = nullptr;
   c->pin_bytes = 0;
@@ -238,13 +248,28 @@ double binom(int n, int k) {
   return r;
 }
 
-// Reads the device error word and maps it to a status (synchronises).
-int check_device(swcs_ctx* c, const char* where) {
+// Enqueues the copy of the status head that check_device waits for, ahead of other copies of the call.
+int read_status(swcs_ctx* c) {
+  int r = ensure_pinned(c, kPinStatus);
+  if (r) return r;
+  CK(cudaMemcpyAsync(c->pin, static_cast<Status*>(ctrl(c)), sizeof(Status), cudaMemcpyDeviceToHost, c->st));
+  return SWCS_OK;
+}
+
+// Waits for the stream, reads the status head (one copy for the error word, the state size and the energies) and maps
+// the error word to a status.  status_read: read_status has been called for it.
+int check_device(swcs_ctx* c, const char* where, bool status_read = false) {
+  int r;
+  if (!status_read && (r = read_status(c))) return r;
   cudaError_t e = cudaStreamSynchronize(c->st);
   if (e != cudaSuccess) return cuda_fail(c, e, where);
-  int derr = 0;
-  CK(cudaMemcpy(&derr, &ctrl(c)->err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (derr == 0) return SWCS_OK;
+  c->pin_busy = false;
+  const Status& s = *(const Status*)c->pin;
+  const int derr = s.err;
+  if (derr == 0) {
+    if (c->have_state) c->n_state_host = s.n_state;
+    return SWCS_OK;
+  }
   int zero = 0;
   CK(cudaMemcpy(&ctrl(c)->err, &zero, sizeof(int), cudaMemcpyHostToDevice));
   c->have_state = false;
@@ -252,6 +277,8 @@ int check_device(swcs_ctx* c, const char* where) {
   if (derr == kDevTableFull) return fail(c, SWCS_ERR_TABLE_FULL, "%s: a device hash table or buffer overflowed", where);
   return fail(c, SWCS_ERR_CUDA, "%s: device reported error %d", where, derr);
 }
+
+const Status& host_status(const swcs_ctx* c) { return *(const Status*)c->pin; }
 
 HamDev ham_dev(swcs_ctx* c) {
   HamDev H;
@@ -587,15 +614,16 @@ int upload_ops(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, int n_o
   if ((r = ensure(c, c->ops_dev, (size_t)5 * n_ops + 16))) return r;
   if ((r = ensure(c, c->cs_dev, (size_t)16 * n_ops + 16))) return r;
   const size_t nb = (size_t)5 * n_ops, cb = (size_t)16 * n_ops;
-  if ((r = ensure_pinned(c, nb + cb + 64))) return r;
-  CK(cudaStreamSynchronize(c->st));  // staging buffer reuse
-  uint8_t* p = (uint8_t*)c->pin;
+  if ((r = ensure_pinned(c, kPinStatus + nb + cb + 64))) return r;
+  if (c->pin_busy) CK(cudaStreamSynchronize(c->st));  // staging buffer reuse
+  uint8_t* p = (uint8_t*)c->pin + kPinStatus;
   double* cs = (double*)(p + ((nb + 15) & ~(size_t)15));
   memcpy(p, h_ops, nb);
   for (int g = 0; g < n_ops; ++g) {  // host cos/sin: one libm call per gate
     cs[2 * g] = std::cos(h_theta[g]);
     cs[2 * g + 1] = std::sin(h_theta[g]);
   }
+  c->pin_busy = true;
   CK(cudaMemcpyAsync(c->ops_dev.p, p, nb, cudaMemcpyHostToDevice, c->st));
   CK(cudaMemcpyAsync(c->cs_dev.p, cs, cb, cudaMemcpyHostToDevice, c->st));
   return SWCS_OK;
@@ -747,23 +775,21 @@ int sweep_rows(swcs_ctx* c, double* d_g, int64_t nd_bound = -1, bool enqueue = t
   CK(cudaMemsetAsync(c->atab.p, 0xff, acap * sizeof(IdxSlot), c->st));
   CK(cudaMemsetAsync(c->gcount.p, 0, nd * 8 + 8, c->st));
   CK(cudaMemsetAsync(c->gfill.p, 0, nd * 8 + 8, c->st));
-  CK(cudaMemsetAsync(&k->n_distinct, 0, 8, c->st));
-  CK(cudaMemsetAsync(k->acc, 0, 16, c->st));
+  CK(cudaMemsetAsync(k->acc, 0, kSweepClear, c->st));
   if (!energy_only && !probe) CK(cudaMemsetAsync(d_g, 0, sizeof(double) * c->pool_size, c->st));
   CK(cudaMemsetAsync(c->rows.p, 0, (size_t)ncl * ((c->NB + 3) & ~(int64_t)3) * 8, c->st));  // rows padded to 32 B
   const GroupArgs ga = group_args(c, acap);
-  CK(launch_k(c, kKGroup, [&] { return launch_group_state(ga, c->st); }));
+  CK(launch_k(c, kKGroup, [&] { return launch_group_state(ga, nd, c->st); }));
   c->launches += 4;  // five grouping kernels in one call
   // beta-single entries carry the spatial pair i * m + j too when ranks fit 21 bits and pairs 10
   const int rbeta_packed = c->NB <= (1 << 21) && m <= 32 ? 1 : 0;
   CK(launch_k(c, kKGroup, [&] {
-    return launch_rbeta(ga.gkey, ga.n, ga.rank_tab, ks, nvs, m, rbeta_packed, (uint32_t*)c->rbeta.p, c->st);
+    return launch_rbeta(ga.gkey, ga.n, ga.rank_tab, ks, nvs, m, rbeta_packed, (uint32_t*)c->rbeta.p, nd, c->st);
   }));
   RowArgs ra = row_args(c, ga, d_g, max_s, max_d, twords, rbeta_packed);
   ra.stage_ent_s = st_s;
   ra.stage_ent_d = st_d;
   ra.target_ctr = &k->row_next;
-  CK(cudaMemsetAsync(&k->row_next, 0, sizeof(unsigned), c->st));
   ra.sel_bits = sel;
   ra.energy_only = energy_only ? 1 : 0;
   ra.sig_out = sig_out;
@@ -816,7 +842,7 @@ int pair_args(swcs_ctx* c, int64_t nd, bool energy, PairArgs* out) {
   a.acc = k->acc;
   a.err = &k->err;
   CK(cudaMemsetAsync(c->pr_tab.p, 0xff, 2 * tcap * sizeof(PairSlot), c->st));
-  CK(cudaMemsetAsync(k->acc, 0, sizeof(k->acc) + sizeof(PairCtl), c->st));
+  CK(cudaMemsetAsync(k->acc, 0, kSweepClear, c->st));
   *out = a;
   return SWCS_OK;
 }
@@ -1324,10 +1350,6 @@ static int apply_common(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta
   if ((r = ensure_state_buffers(c, ms))) return r;
   if (n_ops == 0 && !reset) return SWCS_OK;
   if ((r = upload_ops(c, h_ops, h_theta, n_ops))) return r;
-  if (reset) {
-    long long one = 1;
-    CK(cudaMemcpyAsync(&ctrl(c)->n_state, &one, 8, cudaMemcpyHostToDevice, c->st));
-  }
   if (n_ops == 0) {  // reference determinant only
     const uint8_t id[5] = {0, 0, 0, 0, 0};
     const double z = 0.0;
@@ -1390,11 +1412,9 @@ int swcs_energy_dev(swcs_ctx* c, double* d_out) {
 int swcs_energy(swcs_ctx* c, double* e_out, double* n2_out) {
   int r = swcs_energy_dev(c, nullptr);
   if (r) return r;
-  double out[2];
-  CK(cudaMemcpyAsync(out, ctrl(c)->eout, 16, cudaMemcpyDeviceToHost, c->st));
   if ((r = check_device(c, "swcs_energy"))) return r;
-  if (e_out) *e_out = out[0];
-  if (n2_out) *n2_out = out[1];
+  if (e_out) *e_out = host_status(c).eout[0];
+  if (n2_out) *n2_out = host_status(c).eout[1];
   return SWCS_OK;
 }
 
@@ -1450,16 +1470,17 @@ int swcs_pool_gradients(swcs_ctx* c, double* h_g_out, const int64_t* h_subset, i
   if (!h_g_out) return fail(c, SWCS_ERR_INVALID_ARG, "null output");
   if ((r = ensure(c, c->gdev, sizeof(double) * c->pool_size))) return r;
   if ((r = sweep(c, (double*)c->gdev.p))) return r;
-  if ((r = check_device(c, "swcs_pool_gradients"))) return r;
+  if ((r = read_status(c))) return r;
   if (!h_subset) {
-    CK(cudaMemcpy(h_g_out, c->gdev.p, sizeof(double) * c->pool_size, cudaMemcpyDeviceToHost));
-  } else {
-    std::vector<double> all(c->pool_size);
-    CK(cudaMemcpy(all.data(), c->gdev.p, sizeof(double) * c->pool_size, cudaMemcpyDeviceToHost));
-    for (int64_t i = 0; i < n_subset; ++i) {
-      if (h_subset[i] < 0 || h_subset[i] >= c->pool_size) return fail(c, SWCS_ERR_INVALID_ARG, "subset index out of range");
-      h_g_out[h_subset[i]] = all[h_subset[i]];
-    }
+    CK(cudaMemcpyAsync(h_g_out, c->gdev.p, sizeof(double) * c->pool_size, cudaMemcpyDeviceToHost, c->st));
+    return check_device(c, "swcs_pool_gradients", true);
+  }
+  std::vector<double> all(c->pool_size);
+  CK(cudaMemcpyAsync(all.data(), c->gdev.p, sizeof(double) * c->pool_size, cudaMemcpyDeviceToHost, c->st));
+  if ((r = check_device(c, "swcs_pool_gradients", true))) return r;
+  for (int64_t i = 0; i < n_subset; ++i) {
+    if (h_subset[i] < 0 || h_subset[i] >= c->pool_size) return fail(c, SWCS_ERR_INVALID_ARG, "subset index out of range");
+    h_g_out[h_subset[i]] = all[h_subset[i]];
   }
   return SWCS_OK;
 }
@@ -1575,11 +1596,9 @@ int swcs_stats(swcs_ctx* c, int64_t* out8) {
 int swcs_sweep_energy(swcs_ctx* c, double* e_out, double* n2_out) {
   int r = need_nonempty(c);
   if (r) return r;
-  double out[2];
-  CK(cudaMemcpyAsync(out, ctrl(c)->eout, 16, cudaMemcpyDeviceToHost, c->st));
   if ((r = check_device(c, "swcs_sweep_energy"))) return r;
-  if (e_out) *e_out = out[0];
-  if (n2_out) *n2_out = out[1];
+  if (e_out) *e_out = host_status(c).eout[0];
+  if (n2_out) *n2_out = host_status(c).eout[1];
   return SWCS_OK;
 }
 
@@ -1923,13 +1942,11 @@ int swcs_energy_grad(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, i
   CK(launch_k(c, kKOther, [&] { return launch_scale_dtheta((double*)c->dth.p, n_ops, k->acc, c->st); }));
   CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(k->acc, k->eout, c->st); }));
   if (ncp > 1 && (r = load_slot(ncp))) return r;
-  double out[2];
-  unsigned long long zeros = 0;
-  CK(cudaMemcpyAsync(out, k->eout, 16, cudaMemcpyDeviceToHost, c->st));
-  CK(cudaMemcpyAsync(&zeros, &k->zeros, 8, cudaMemcpyDeviceToHost, c->st));
+  if ((r = read_status(c))) return r;
   if (h_dtheta_out) CK(cudaMemcpyAsync(h_dtheta_out, c->dth.p, (size_t)n_ops * 8, cudaMemcpyDeviceToHost, c->st));
-  if ((r = check_device(c, "swcs_energy_grad"))) return r;
-  if (h_e_out) *h_e_out = out[0];
+  if ((r = check_device(c, "swcs_energy_grad", true))) return r;
+  if (h_e_out) *h_e_out = host_status(c).eout[0];
+  const bool zeros = host_status(c).zeros != 0;
   // leave psi_M as the context's state: an identity pass rebuilds the index after replays and drops the zero
   // amplitudes that the projectors kept
   if (ncp > 1 || zeros) {

@@ -185,7 +185,8 @@ size_t row_sweep_smem(int max_ent_s, int max_ent_d, int stage_ent_s, int stage_e
 cudaError_t row_sweep_max_clusters(int threads, int occ, int gsz, size_t smem, int* n_clusters);
 cudaError_t launch_row_sweep(const RowArgs& a, int threads, int occ, int gsz, int n_clusters, size_t smem,
                              cudaStream_t st);
-cudaError_t launch_group_state(const GroupArgs& g, cudaStream_t st);
+// n_max: at least the number of determinants (sizes the grids).
+cudaError_t launch_group_state(const GroupArgs& g, int64_t n_max, cudaStream_t st);
 // State of the top-N radix select (gate kernel: every CTA keeps an identical copy in shared memory;
 // batched kernel: one copy per instance in global memory).
 struct SelState {
@@ -255,7 +256,7 @@ cudaError_t launch_batch(const BatchInst* d_inst, BatchSched* d_sched, int n_ins
 cudaError_t launch_screen_lists(const int* kab, int m, const uint32_t* sel_bits, int* ab_cnt, uint2* ab_list,
                                 cudaStream_t st);
 cudaError_t launch_rbeta(const uint64_t* gkey, const long long* n, const uint32_t* rank_tab, int ks, int nv, int m,
-                         int packed, uint32_t* rbeta, cudaStream_t st);
+                         int packed, uint32_t* rbeta, int64_t n_max, cudaStream_t st);
 
 // Adjoint (swcs_adjoint.cu).
 cudaError_t launch_build_index(const uint64_t* keys, const long long* n, IdxSlot* tab, uint64_t mask, cudaStream_t st);

@@ -142,6 +142,10 @@ __global__ void screen_lists_kernel(const int* kab, int m, const uint32_t* sel_b
 
 }  // namespace
 
+// 256-thread CTAs for n items, up to the whole device: a launch of 1,216 CTAs for a handful of determinants costs
+// more than their work.
+static int grid_for(int64_t n) { return (int)(n < 1 ? 1 : n < (int64_t)1216 * 256 ? (n + 255) / 256 : 1216); }
+
 cudaError_t launch_screen_lists(const int* kab, int m, const uint32_t* sel_bits, int* ab_cnt, uint2* ab_list,
                                 cudaStream_t st) {
   screen_lists_kernel<<<m * m, 256, 0, st>>>(kab, m, sel_bits, ab_cnt, ab_list);
@@ -149,8 +153,8 @@ cudaError_t launch_screen_lists(const int* kab, int m, const uint32_t* sel_bits,
 }
 
 cudaError_t launch_rbeta(const uint64_t* gkey, const long long* n, const uint32_t* rank_tab, int ks, int nv, int m,
-                         int packed, uint32_t* rbeta, cudaStream_t st) {
-  rbeta_kernel<<<1216, 256, 0, st>>>(gkey, n, rank_tab, ks, nv, m, packed, rbeta);
+                         int packed, uint32_t* rbeta, int64_t n_max, cudaStream_t st) {
+  rbeta_kernel<<<grid_for(32 * n_max), 256, 0, st>>>(gkey, n, rank_tab, ks, nv, m, packed, rbeta);
   return cudaGetLastError();
 }
 
@@ -224,10 +228,10 @@ cudaError_t launch_row_sweep(const RowArgs& a, int threads, int occ, int gsz, in
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_group_state(const GroupArgs& g, cudaStream_t st) {
-  const int nb = 1216;
+cudaError_t launch_group_state(const GroupArgs& g, int64_t n_max, cudaStream_t st) {
+  const int nb = grid_for(n_max);
   group_insert_kernel<<<nb, 256, 0, st>>>(g.keys, g.n, g.atab, g.amask, g.amps, g.acc);
-  group_ids_kernel<<<nb, 256, 0, st>>>(g.atab, g.amask + 1, g.n_groups);
+  group_ids_kernel<<<grid_for((int64_t)g.amask + 1), 256, 0, st>>>(g.atab, g.amask + 1, g.n_groups);
   group_count_kernel<<<nb, 256, 0, st>>>(g.keys, g.n, g.atab, g.amask, g.gid_of, g.gcount);
   group_scan_kernel<<<1, 1024, 0, st>>>(g.gcount, g.n_groups, g.goff);
   group_scatter_kernel<<<nb, 256, 0, st>>>(g.keys, g.amps, g.n, g.gid_of, g.goff, g.gfill, g.gkey, g.gamp, g.grank,
