@@ -23,6 +23,18 @@ namespace {
 
 constexpr uint64_t kTimeoutNs = 2000000000ull;  // bounded device waits: 2 s
 
+// Work arrays of the in-place gate sequence, in one allocation: a context's first gates paid for nine.
+struct GateMem {
+  uint64_t* keys;
+  double* amps[2];
+  uint64_t* low_keys;
+  double* low_amps;
+  BandEntry* band_ent;
+  uint32_t* ring;
+  unsigned* band;
+  uint32_t* low_rec;
+};
+
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
@@ -79,7 +91,8 @@ struct swcs_ctx {
   int opt_row_clusters = 0;  // clusters of the row sweep (0: as many as fit)
 
   // in-place gate sequence: second amplitude array, partners put aside, free positions, positions of the output
-  DevBuf amps_c, low_keys, low_amps, low_rec, ring, out_pos, band, band_slots;
+  DevBuf gate_mem, out_pos;
+  GateMem gm{};  // the pieces of gate_mem
   DevBuf sort_k1, sort_v1, sort_k2, sort_v2, sort_cnt;  // copy-out in bitstring order
   int64_t max_state = 0;    // determinants the state buffers are sized for
   int cluster_ok[17] = {};  // clusters of k gate CTAs: 0 unknown, 1 fit, -1 do not
@@ -382,8 +395,6 @@ int ensure_state_buffers(swcs_ctx* c, int64_t max_state) {
     release(c->amps_a);
     c->keys_a = nk;
     c->amps_a = na;
-    if ((r = ensure(c, c->keys_b, cap * 8))) return r;
-    if ((r = ensure(c, c->amps_b, cap * 8))) return r;
     if ((r = ensure(c, c->tab0, tcap * sizeof(IdxSlot)))) return r;
     if ((r = ensure(c, c->tab1, tcap * sizeof(IdxSlot)))) return r;
     c->cap = cap;
@@ -401,13 +412,24 @@ int band_slots_for(int64_t max_state) { return max_state <= 16384 ? 8 : 32; }
 // (tab1 as 8-byte slots: at least 4 N) holds the determinants kept and dropped ones' slots until it is built anew.
 int ensure_gate_buffers(swcs_ctx* c) {
   const size_t n = (size_t)c->max_state, np = 4 * n + 64;
-  int r;
-  if ((r = ensure(c, c->keys_b, np * 8)) || (r = ensure(c, c->amps_b, np * 8)) || (r = ensure(c, c->amps_c, np * 8)) ||
-      (r = ensure(c, c->low_keys, n * 8)) || (r = ensure(c, c->low_amps, n * 8)) || (r = ensure(c, c->low_rec, n * 4)) ||
-      (r = ensure(c, c->ring, pow2_at_least(np) * 4)) || (r = ensure(c, c->band, 3 * kBandWords * 4)) ||
-      (r = ensure(c, c->band_slots, (size_t)3 * kBandBins * band_slots_for(c->max_state) * sizeof(BandEntry))))
-    return r;
+  const size_t sizes[] = {np * 8, np * 8, np * 8, n * 8, n * 8,
+                          (size_t)3 * kBandBins * band_slots_for(c->max_state) * sizeof(BandEntry),
+                          pow2_at_least(np) * 4, 3 * kBandWords * 4, n * 4};
+  size_t at[10] = {0};
+  for (int i = 0; i < 9; ++i) at[i + 1] = at[i] + ((sizes[i] + 255) & ~(size_t)255);
+  const int r = ensure(c, c->gate_mem, at[9]);
+  if (r) return r;
+  char* p = (char*)c->gate_mem.p;
+  c->gm = {(uint64_t*)(p + at[0]), {(double*)(p + at[1]), (double*)(p + at[2])}, (uint64_t*)(p + at[3]),
+           (double*)(p + at[4]), (BandEntry*)(p + at[5]), (uint32_t*)(p + at[6]), (unsigned*)(p + at[7]),
+           (uint32_t*)(p + at[8])};
   return SWCS_OK;
+}
+
+// Second copy of the state, for the rebuilding gate kernel only.
+int ensure_rebuild_buffers(swcs_ctx* c) {
+  const int r = ensure(c, c->keys_b, c->cap * 8);
+  return r ? r : ensure(c, c->amps_b, c->cap * 8);
 }
 
 constexpr int64_t kMaxInPlace = (int64_t)1 << 28;  // positions (four times that) fit 31 bits
@@ -505,19 +527,19 @@ int run_gates(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, 
     a.in_amps = (const double*)c->amps_a.p;
     a.out_keys = (uint64_t*)c->keys_a.p;
     a.out_amps = (double*)c->amps_a.p;
-    a.keys = (uint64_t*)c->keys_b.p;
-    a.amp[0] = (double*)c->amps_b.p;
-    a.amp[1] = (double*)c->amps_c.p;
+    a.keys = c->gm.keys;
+    a.amp[0] = c->gm.amps[0];
+    a.amp[1] = c->gm.amps[1];
     a.cap = (uint32_t)(4 * c->max_state + 64);
     a.tab = (uint64_t*)c->tab1.p;
     a.tab_mask = 2 * c->tab_mask + 1;
     a.plain = (IdxSlot*)c->tab0.p;
     a.plain_mask = c->tab_mask;
-    a.low_keys = (uint64_t*)c->low_keys.p;
-    a.low_amps = (double*)c->low_amps.p;
-    a.low_rec = (uint32_t*)c->low_rec.p;
+    a.low_keys = c->gm.low_keys;
+    a.low_amps = c->gm.low_amps;
+    a.low_rec = c->gm.low_rec;
     a.cap_low = (uint32_t)c->max_state;
-    a.ring = (uint32_t*)c->ring.p;
+    a.ring = c->gm.ring;
     a.ring_mask = (uint32_t)(pow2_at_least(4 * (uint64_t)c->max_state + 64) - 1);
     a.ops = d_ops;
     a.cs = d_cs;
@@ -529,8 +551,8 @@ int run_gates(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, 
     a.n_state = &k->n_state;
     a.ctr = k->gate_ctr;
     a.hist = (unsigned*)c->selhist.p;
-    a.band = (unsigned*)c->band.p;
-    a.band_ent = (BandEntry*)c->band_slots.p;
+    a.band = c->gm.band;
+    a.band_ent = c->gm.band_ent;
     a.band_slots = band_slots_for(c->max_state);
     a.bar = &k->bar;
     a.err = &k->err;
@@ -556,6 +578,7 @@ int run_gates(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, 
   const int gthreads = c->opt_gate_threads;
   const int bps = ansatz_blocks_per_sm(gthreads);
   if (bps <= 0) return fail(c, SWCS_ERR_NO_DEVICE, "ansatz kernel cannot be resident on this device");
+  if ((r = ensure_rebuild_buffers(c))) return r;
   const AnsatzArgs a = gate_args(c, d_ops, d_cs, n_ops, n_keep, reset);
   CK(cudaMemsetAsync(&k->bar, 0, sizeof(GridBar), c->st));
   int nblocks = c->nsm * bps;
@@ -1073,8 +1096,7 @@ int swcs_destroy(swcs_ctx* c) {
                     &c->gid_of, &c->gcount, &c->goff, &c->gfill, &c->gkey, &c->gamp, &c->grank, &c->rows,
                     &c->rbeta, &c->gab, &c->kab, &c->gorig,
                     &c->ck_keys, &c->ck_amps, &c->ck_n, &c->tp_pos, &c->tp_x, &c->tp_drop, &c->tp_start, &c->sigma,
-                    &c->nu0, &c->nu1, &c->atab0, &c->dth, &c->amps_c, &c->low_keys, &c->low_amps, &c->low_rec, &c->ring,
-                    &c->out_pos, &c->band, &c->band_slots, &c->sort_k1, &c->sort_v1, &c->sort_k2, &c->sort_v2, &c->sort_cnt, &c->pool_dev, &c->selbits, &c->feat,
+                    &c->nu0, &c->nu1, &c->atab0, &c->dth, &c->gate_mem, &c->out_pos, &c->sort_k1, &c->sort_v1, &c->sort_k2, &c->sort_v2, &c->sort_cnt, &c->pool_dev, &c->selbits, &c->feat,
                     &c->ypred, &c->topk_hist, &c->topk_ctl, &c->occ, &c->prb, &c->ab_cnt, &c->ab_list,
                     &c->selhist, &c->pr_tab, &c->pr_slot, &c->pr_pos, &c->pr_rec, &c->pr_oth, &c->pr_idx, &c->pr_items,
                     &c->rdm_tab, &c->rdm_work, &c->rdm_gamma};
@@ -2259,7 +2281,7 @@ int swcs_batch_add(swcs_batch* b, const double* h_h, const double* h_g, int n_so
   if ((r = validate_ops(c, h_ops, n_ops))) return undo(r);
   const int64_t ms = max_state_for(c, n_keep, n_ops, 1);
   if (ms > ((int64_t)1 << 31)) return undo(fail(c, SWCS_ERR_INVALID_ARG, "state bound too large: give n_keep"));
-  if ((r = ensure_state_buffers(c, ms)) || (r = upload_ops(c, h_ops, h_theta, n_ops)) ||
+  if ((r = ensure_state_buffers(c, ms)) || (r = ensure_rebuild_buffers(c)) || (r = upload_ops(c, h_ops, h_theta, n_ops)) ||
       (r = ensure(c, c->gdev, sizeof(double) * c->pool_size)))
     return undo(r);
   if (cudaStreamSynchronize(st) != cudaSuccess) return undo(SWCS_ERR_CUDA);
