@@ -1,7 +1,10 @@
 // Batched persistent launch (the many-instances workload): one kernel runs
 // every instance's whole hot path -- the gate sequence of Eq. 1 with merge and
 // truncation after every gate (Sec. II.B), then the pool sweep of ADAPT step 4
-// (Sec. II.C) -- for all instances at once.
+// (Sec. II.C) -- for all instances at once.  Instances whose sweep is faster
+// through the density matrices (swcs_rdm.cu) get it as a chain of launches in
+// the same graph, and their gates too as a launch beside this kernel or, for
+// very large states, in here (BatchInst::n_mat: no row phases).
 //
 // Work items are (instance, phase, tile).  Each instance walks a chain of
 // phases (BatchPhase): initial index tables; per gate the gate pass (which also
@@ -356,6 +359,10 @@ __device__ void epilogue(const BatchInst& I, BatchSched& S, const BatchTask& k, 
     if (nx.gate < I.n_ops) {
       nx.type = kPhGate;
       nx.ntiles = max(1u, ceil_div(n_state, tile));
+    } else if (I.n_mat) {  // its sweep follows this kernel
+      nx.type = kPhDone;
+      nx.ntiles = 0;
+      if (threadIdx.x == 0) *I.n_mat = n_state;
     } else {
       nx.type = kPhGroupClear;
       nx.ntiles = ceil_div(max(max((long long)I.acap, (long long)I.pool_size), n_state + 1), tile);

@@ -437,19 +437,19 @@ constexpr int64_t kMaxInPlace = (int64_t)1 << 28;  // positions (four times that
 // CTAs of a gate-sequence or backward launch: up to 16 form one cluster where the device takes such clusters
 // (barriers of a fraction of a microsecond), larger states and launches with test hooks use a cooperative grid.
 // Measured per gate: see swcs_gates.cu.
-void gate_launch_shape(swcs_ctx* c, int per_sm, int* nblocks, bool* clustered) {
+void gate_launch_shape(swcs_ctx* c, int (*per_sm)(), int* nblocks, bool* clustered, bool one_cluster = false) {
   const int64_t want = (c->max_state + 2047) / 2048;
   *clustered = false;
-  if (c->opt_skip_arrive < 0 && c->opt_gate_blocks == 0 && want <= 8) {
+  if (c->opt_skip_arrive < 0 && c->opt_gate_blocks == 0 && (want <= 8 || one_cluster)) {
     const int k = (int)std::max<int64_t>(1, std::min<int64_t>((c->max_state + 1023) / 1024, 16));
-    if (c->cluster_ok[k] == 0) c->cluster_ok[k] = gate_cluster_fits(k) > 0 ? 1 : -1;
+    if (c->cluster_ok[k] == 0) c->cluster_ok[k] = k == 1 || gate_cluster_fits(k) > 0 ? 1 : -1;
     if (c->cluster_ok[k] > 0) {
       *nblocks = k;
       *clustered = true;
       return;
     }
   }
-  int nb = c->nsm * std::max(per_sm, 1);
+  int nb = c->nsm * std::max(per_sm(), 1);
   if (c->opt_gate_blocks > 0) nb = std::min(nb, c->opt_gate_blocks);
   else nb = (int)std::max<int64_t>(std::min<int64_t>(nb, (c->max_state + 511) / 512), std::min(nb, 8));
   *nblocks = nb;
@@ -511,6 +511,7 @@ AnsatzArgs gate_args(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int 
 struct GateRun {
   const GateTape* tape = nullptr;
   bool keep_zeros = false;
+  bool one_cluster = false;  // whatever the size of the state
 };
 
 // The gate sequence, in place (swcs_gates.cu).  Instances that share the device (batch mode 1, captured) and states
@@ -566,7 +567,7 @@ int run_gates(swcs_ctx* c, const uint8_t* d_ops, const double* d_cs, int n_ops, 
     }
     int nblocks = 0;
     bool clustered = false;
-    gate_launch_shape(c, gate_blocks_per_sm(), &nblocks, &clustered);
+    gate_launch_shape(c, gate_blocks_per_sm, &nblocks, &clustered, run.one_cluster);
     if (!clustered) CK(cudaMemsetAsync(&k->bar, 0, sizeof(GridBar), c->st));  // barrier words must start at zero
     CK(launch_k(c, kKAnsatz, [&] { return launch_gates(a, nblocks, clustered, c->st); }));
     c->tab_cur = 0;
@@ -903,50 +904,71 @@ int energy_rows(swcs_ctx* c, double* sig_out) {
 //             that of full matrices (m^7).  A determinant of such states has some 300 neighbours within three
 //             excitations; one that fills a share of the sector has that share of all of them (1.5 times, as
 //             states crowd around the reference).
+struct SweepCost {
+  double rows, mats;  // us
+};
+
+SweepCost sweep_cost(swcs_ctx* c, int64_t nd) {
+  const double n = (double)nd, m = c->n / 2, no = c->no, nv = c->nv;
+  const double single = no * nv, dbl = binom(c->no, 2) * binom(c->nv, 2), triple = binom(c->no, 3) * binom(c->nv, 3);
+  const double conn = 2.0 * single + 2.0 * dbl + single * single;
+  const double three = conn + 2.0 * triple + 2.0 * dbl * single;
+  const double hits = 300.0 + 1.5 * n / c->fci_dim * three;
+  return {60.0 + 0.008 * c->NA + 2.0 * n * (conn + 1.0) / 1.18e5,
+          110.0 + (double)rdm_gamma_doubles(c->n / 2) * 8.0 / 2.1e6 + 740.0 * std::pow(m / 26.0, 6) +
+              n * (0.008 + hits / 9.6e4) + std::min(1070.0 * std::pow(m / 14.0, 7), 0.025 * n)};
+}
+
 bool use_density_matrices(swcs_ctx* c, int64_t nd) {
   if (c->opt_sweep != 0 || c->opt_count_probes || c->opt_pairs == 0) return false;
   if (c->no < 2 || nd > kMaxPairDets) return false;
   if (c->opt_pairs == 1) return true;
   if (c->NB <= 0 || c->NB > (1 << 22)) return true;  // no row sweep there: the hashed table is slower than either
-  const double n = (double)nd, m = c->n / 2, no = c->no, nv = c->nv;
-  const double single = no * nv, dbl = binom(c->no, 2) * binom(c->nv, 2), triple = binom(c->no, 3) * binom(c->nv, 3);
-  const double conn = 2.0 * single + 2.0 * dbl + single * single;
-  const double three = conn + 2.0 * triple + 2.0 * dbl * single;
-  const double rows = 60.0 + 0.008 * c->NA + 2.0 * n * (conn + 1.0) / 1.18e5;
-  const double hits = 300.0 + 1.5 * n / c->fci_dim * three;
-  const double mats = 110.0 + (double)rdm_gamma_doubles(c->n / 2) * 8.0 / 2.1e6 + 740.0 * std::pow(m / 26.0, 6) +
-                      n * (0.008 + hits / 9.6e4) + std::min(1070.0 * std::pow(m / 14.0, 7), 0.025 * n);
-  return mats < rows;
+  const SweepCost t = sweep_cost(c, nd);
+  return t.mats < t.rows;
 }
 
-// Pool gradient and energy from the density matrices (swcs_rdm.cu); 1 when their memory cannot be had.
-int sweep_density(swcs_ctx* c, double* d_g, int64_t nd) {
+// The Hamiltonian's tables for the density-matrix sweep, once per Hamiltonian, from its staged copy.
+int ensure_rdm_tables(swcs_ctx* c) {
+  const int m = c->n / 2, r = ensure(c, c->rdm_tab, rdm_table_doubles(m) * 8);
+  if (r || c->rdm_tables_ready) return r;
+  CK(launch_k(c, kKOther, [&] {
+    return launch_rdm_tables((const double*)c->gstage.p, c->n, rdm_tables((double*)c->rdm_tab.p, m), c->st);
+  }));
+  c->rdm_tables_ready = true;
+  return SWCS_OK;
+}
+
+// The density-matrix sweep itself: up to nd determinants, *d_n of them (nullptr: the context's state), over the
+// given matrices and work space; enqueues only, apart from pair buffers that are not there yet.
+int enqueue_density(swcs_ctx* c, double* d_g, int64_t nd, const long long* d_n, double* gamma, double* work) {
   const int m = c->n / 2;
-  const size_t gd = rdm_gamma_doubles(m);
-  if (ensure(c, c->rdm_gamma, gd * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8) ||
-      ensure(c, c->rdm_tab, rdm_table_doubles(m) * 8))
-    return 1;
-  if (!c->rdm_tables_ready) {  // once per Hamiltonian, from its staged copy
-    CK(launch_k(c, kKOther, [&] {
-      return launch_rdm_tables((const double*)c->gstage.p, c->n, rdm_tables((double*)c->rdm_tab.p, m), c->st);
-    }));
-    c->rdm_tables_ready = true;
-  }
   RdmArgs a{};
   const int r = pair_args(c, nd, false, &a.P);
   if (r) return r;
-  rdm_layout(a, (double*)c->rdm_work.p, (double*)c->rdm_gamma.p, m);
+  if (d_n) a.P.n = d_n;
+  rdm_layout(a, work, gamma, m);
   a.V = rdm_tables((double*)c->rdm_tab.p, m);
   a.pool_ops = (const uint8_t*)c->pool_dev.p;
   a.pool_size = c->pool_size;
   a.g = d_g;
-  CK(cudaMemsetAsync(c->rdm_gamma.p, 0, gd * 8, c->st));
+  CK(cudaMemsetAsync(gamma, 0, rdm_gamma_doubles(m) * 8, c->st));
   CK(launch_k(c, kKGroup, [&] { return launch_pairs_gamma(a.P, nd, c->nsm, c->st); }));
   CK(launch_k(c, kKRow, [&] { return launch_rdm_gradient(a, c->nsm, c->st); }));
   c->launches += 4 + (c->no >= 3 ? 8 : 7);
   CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(ctrl(c)->acc, ctrl(c)->eout, c->st); }));
   c->stats[2] = c->stats[3] = c->stats[4] = 0;
   return SWCS_OK;
+}
+
+// Pool gradient and energy from the density matrices (swcs_rdm.cu); 1 when their memory cannot be had.
+int sweep_density(swcs_ctx* c, double* d_g, int64_t nd) {
+  const int m = c->n / 2;
+  if (ensure(c, c->rdm_gamma, rdm_gamma_doubles(m) * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8) ||
+      ensure(c, c->rdm_tab, rdm_table_doubles(m) * 8))
+    return 1;
+  const int r = ensure_rdm_tables(c);
+  return r ? r : enqueue_density(c, d_g, nd, nullptr, (double*)c->rdm_gamma.p, (double*)c->rdm_work.p);
 }
 
 int sweep(swcs_ctx* c, double* d_g, const uint32_t* sel = nullptr) {
@@ -1933,7 +1955,7 @@ int swcs_energy_grad(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, i
   // ---- backward, one segment at a time: the segment's tape again, nu brought to its last positions by key
   int cur = 0, nblocks = 0;
   bool clustered = false;
-  gate_launch_shape(c, back_blocks_per_sm(), &nblocks, &clustered);
+  gate_launch_shape(c, back_blocks_per_sm, &nblocks, &clustered);
   for (int seg = ncp - 1; seg >= 0; --seg) {
     const int g0 = seg * ck, g1 = std::min(n_ops, g0 + ck);
     if (seg < ncp - 1) {
@@ -1985,6 +2007,10 @@ int swcs_energy_grad(swcs_ctx* c, const uint8_t* h_ops, const double* h_theta, i
 // =============================================================================
 // Batched launch: many independent instances in one CUDA graph.
 // =============================================================================
+namespace {
+constexpr int kBatchLanes = 4;
+}
+
 struct swcs_batch {
   cudaStream_t origin = nullptr;
   bool own_origin = false;  // created here: the legacy default stream cannot be captured
@@ -2011,6 +2037,10 @@ struct swcs_batch {
   int* d_status = nullptr;
   size_t rows_bytes = 0, inst_bytes = 0;
   int nblocks = 0;
+  // density-matrix sweeps after the persistent kernel: their state sizes and each lane's matrices and work space
+  int n_kernel = 0;  // instances inside the persistent kernel
+  long long* d_nmat = nullptr;
+  double* lane_mem[kBatchLanes] = {};
   uint64_t timeout_ns = kTimeoutNs;  // bound of the persistent kernel's wait for work
   int stall_instance = -1;           // test hook: this instance's first phase is never picked up
 };
@@ -2089,8 +2119,14 @@ int batch_capture(swcs_batch* b, double share, int cluster) {
 }
 
 void batch_free_persistent(swcs_batch* b) {
-  for (void* p : {(void*)b->d_inst, (void*)b->d_sched, (void*)b->d_sched0, (void*)b->d_rows, (void*)b->d_status})
+  for (void* p : {(void*)b->d_inst, (void*)b->d_sched, (void*)b->d_sched0, (void*)b->d_rows, (void*)b->d_status,
+                  (void*)b->d_nmat})
     if (p) cudaFree(p);
+  for (double*& p : b->lane_mem) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  }
+  b->d_nmat = nullptr;
   b->d_inst = nullptr;
   b->d_sched = b->d_sched0 = nullptr;
   b->d_rows = nullptr;
@@ -2098,16 +2134,81 @@ void batch_free_persistent(swcs_batch* b) {
   b->rows_bytes = b->inst_bytes = 0;
 }
 
+// How the instances run.  lane[i] < 0: gates and row sweep inside the persistent kernel.  Otherwise the sweep goes
+// through the density matrices (the single context's rule, at the instance's bound on its state), in one of
+// kBatchLanes chains beside the kernel, whose instances share the chain's matrices; and own[i]: its gates are a launch
+// of their own too, one cluster of up to 16 CTAs, so its sweep need not wait for the other instances' gates (states
+// of more than kClusterDets determinants are too much work for one cluster).  Twelve instances of 16 to 38
+// spin-orbitals and up to 76,000 determinants, four of them by chains: 20.5 ms with everything in the kernel (a gate
+// takes 60 us there, phase by phase), 17.6 ms with the four sweeps as chains after it, 10.4 ms with their gates beside
+// it too.  Without memory for the matrices every instance goes by rows.
+constexpr int64_t kClusterDets = 131072;
+
+int batch_plan_density(swcs_batch* b, std::vector<int>& lane, std::vector<char>& own) {
+  const int n = (int)b->inst.size();
+  lane.assign(n, -1);
+  own.assign(n, 0);
+  std::vector<std::pair<double, int>> todo;
+  for (int i = 0; i < n; ++i)
+    if (i != b->stall_instance && use_density_matrices(b->inst[i], b->max_state[i]))
+      todo.push_back({sweep_cost(b->inst[i], b->max_state[i]).mats, i});
+  if (todo.empty()) return SWCS_OK;
+  std::sort(todo.begin(), todo.end(), [](auto& x, auto& y) { return x.first > y.first; });
+  double load[kBatchLanes] = {};
+  size_t need[kBatchLanes] = {};
+  for (auto& [t, i] : todo) {
+    const int l = (int)(std::min_element(load, load + kBatchLanes) - load), m = b->inst[i]->n / 2;
+    load[l] += t;
+    need[l] = std::max(need[l], rdm_gamma_doubles(m) + rdm_work_doubles(m));
+    lane[i] = l;
+  }
+  bool ok = cudaMalloc((void**)&b->d_nmat, n * sizeof(long long)) == cudaSuccess;
+  for (int l = 0; l < kBatchLanes && ok; ++l)
+    ok = !need[l] || cudaMalloc((void**)&b->lane_mem[l], need[l] * 8) == cudaSuccess;
+  for (int i = 0; i < n && ok; ++i) {
+    swcs_ctx* c = b->inst[i];
+    PairArgs a;
+    if (lane[i] < 0) continue;
+    ok = ensure_rdm_tables(c) == SWCS_OK && pair_args(c, b->max_state[i], false, &a) == SWCS_OK;  // its buffers
+    if (ok && cudaStreamSynchronize(c->st) != cudaSuccess) return bfail(b, SWCS_ERR_CUDA, "batch: Hamiltonian tables");
+    if (!ok || b->max_state[i] > kClusterDets || ensure_gate_buffers(c) != SWCS_OK) continue;
+    c->opt_gate_threads = kAnsatzThreads;
+    c->opt_gate_blocks = 0;
+    int k = 0;
+    bool clustered = false;
+    gate_launch_shape(c, gate_blocks_per_sm, &k, &clustered, true);
+    own[i] = clustered;
+  }
+  if (!ok) {
+    cudaGetLastError();
+    lane.assign(n, -1);
+    own.assign(n, 0);
+    if (b->d_nmat) cudaFree(b->d_nmat);
+    b->d_nmat = nullptr;
+    for (double*& p : b->lane_mem) {
+      if (p) cudaFree(p);
+      p = nullptr;
+    }
+  }
+  return SWCS_OK;
+}
+
 // The persistent launch: per-instance descriptors (gate, grouping and row-sweep
 // arguments over the instance's own buffers), the initial scheduler words, and
-// a graph of {scheduler reset, status reset, row reset, the kernel}.
+// a graph of {scheduler reset, status reset, row reset, the kernel} beside the
+// chains of density-matrix sweeps.
 int batch_build_persistent(swcs_batch* b, int tile, int occ, int hash_factor) {
   batch_drop_graph(b);
   const int n = (int)b->inst.size();
-  std::vector<BatchInst> hi(n);
-  std::vector<BatchSched> hs(n);
+  std::vector<BatchInst> hi;
+  std::vector<BatchSched> hs;
   size_t dyn = 0;
   int64_t max_nb = 4;
+  batch_free_persistent(b);
+  std::vector<int> lane;
+  std::vector<char> own;
+  if (const int r = batch_plan_density(b, lane, own)) return r;
+  double t_kernel = 0.0, t_chains = 0.0;
   for (int i = 0; i < n; ++i) {
     swcs_ctx* c = b->inst[i];
     const int m = c->n / 2;
@@ -2123,19 +2224,30 @@ int batch_build_persistent(swcs_batch* b, int tile, int occ, int hash_factor) {
       smem = row_sweep_smem(max_s, max_d, 0, 0, t_same, 0);
     }
     if (smem > 96 * 1024) return bfail(b, SWCS_ERR_INVALID_ARG, "batch: an instance's sector does not fit the row sweep");
-    dyn = std::max(dyn, smem);
-    max_nb = std::max<int64_t>(max_nb, c->NB);
+    const bool rows = lane[i] < 0;
+    const SweepCost cost = sweep_cost(c, nd);
+    if (own[i]) {
+      t_chains += cost.mats;
+      continue;
+    }
+    t_kernel += rows ? cost.rows : 0.0;
+    if (rows) {
+      dyn = std::max(dyn, smem);
+      max_nb = std::max<int64_t>(max_nb, c->NB);
+    }
     const uint64_t acap = pow2_at_least((uint64_t)std::max<int64_t>((int64_t)hash_factor * nd, 64));
     int r;
-    if ((r = ensure(c, c->atab, acap * sizeof(IdxSlot))) || (r = ensure(c, c->gid_of, nd * 4 + 4)) ||
-        (r = ensure(c, c->gcount, nd * 8 + 8)) || (r = ensure(c, c->goff, nd * 8 + 16)) ||
-        (r = ensure(c, c->gfill, nd * 8 + 8)) || (r = ensure(c, c->gkey, nd * 8 + 8)) ||
-        (r = ensure(c, c->gamp, nd * 8 + 8)) || (r = ensure(c, c->grank, nd * 4 + 4)) ||
-        (r = ensure(c, c->rbeta, (size_t)std::max<int64_t>(nd, 1) * ks * nvs * 4)) ||
-        (r = ensure(c, c->gorig, (size_t)std::max<int64_t>(nd, 1) * 4)))
+    if (rows && ((r = ensure(c, c->atab, acap * sizeof(IdxSlot))) || (r = ensure(c, c->gid_of, nd * 4 + 4)) ||
+                 (r = ensure(c, c->gcount, nd * 8 + 8)) || (r = ensure(c, c->goff, nd * 8 + 16)) ||
+                 (r = ensure(c, c->gfill, nd * 8 + 8)) || (r = ensure(c, c->gkey, nd * 8 + 8)) ||
+                 (r = ensure(c, c->gamp, nd * 8 + 8)) || (r = ensure(c, c->grank, nd * 4 + 4)) ||
+                 (r = ensure(c, c->rbeta, (size_t)std::max<int64_t>(nd, 1) * ks * nvs * 4)) ||
+                 (r = ensure(c, c->gorig, (size_t)std::max<int64_t>(nd, 1) * 4))))
       return bfail(b, r, "batch: " + c->err);
     const int packed = c->NB <= (1 << 21) && m <= 32 ? 1 : 0;
-    BatchInst& I = hi[i];
+    hi.emplace_back();
+    BatchInst& I = hi.back();
+    I = BatchInst{};
     I.ga = gate_args(c, (const uint8_t*)c->ops_dev.p, (const double*)c->cs_dev.p, b->n_ops[i], b->n_keep[i], true);
     I.gr = group_args(c, acap);
     I.ra = row_args(c, I.gr, (double*)c->gdev.p, max_s, max_d, twords, packed);
@@ -2149,7 +2261,9 @@ int batch_build_persistent(swcs_batch* b, int tile, int occ, int hash_factor) {
     I.g = (double*)c->gdev.p;
     I.pool_size = c->pool_size;
     I.eout = ctrl(c)->eout;
-    BatchSched& S = hs[i];
+    I.n_mat = rows ? nullptr : b->d_nmat + i;
+    hs.emplace_back();
+    BatchSched& S = hs.back();
     S = BatchSched{};
     S.tab_cur = 0;
     S.ep = 1;
@@ -2162,32 +2276,83 @@ int batch_build_persistent(swcs_batch* b, int tile, int occ, int hash_factor) {
   }
   const int bps = std::min(occ, batch_blocks_per_sm(dyn));
   if (bps <= 0) return bfail(b, SWCS_ERR_NO_DEVICE, "batch: the persistent kernel cannot be resident on this device");
-  const int nblocks = b->inst[0]->nsm * bps;
+  // beside chains the kernel takes its share of the device, by the sweeps' costs; at least a CTA on every fourth SM
+  const int nk = (int)hi.size(), nsm = b->inst[0]->nsm;
+  int nblocks = nsm * bps;
+  if (t_chains > 0.0)
+    nblocks = std::max(std::min(nblocks, (int)std::lround(nblocks * t_kernel / (t_kernel + t_chains))), nsm / 4);
   const int64_t row_stride = (max_nb + 3) & ~(int64_t)3;
   const size_t rows_bytes = (size_t)nblocks * row_stride * 8;
-  batch_free_persistent(b);
-  if (cudaMalloc(&b->d_inst, n * sizeof(BatchInst)) != cudaSuccess ||
-      cudaMalloc((void**)&b->d_sched, n * sizeof(BatchSched)) != cudaSuccess ||
-      cudaMalloc((void**)&b->d_sched0, n * sizeof(BatchSched)) != cudaSuccess ||
+  if (cudaMalloc(&b->d_inst, std::max(nk, 1) * sizeof(BatchInst)) != cudaSuccess ||
+      cudaMalloc((void**)&b->d_sched, std::max(nk, 1) * sizeof(BatchSched)) != cudaSuccess ||
+      cudaMalloc((void**)&b->d_sched0, std::max(nk, 1) * sizeof(BatchSched)) != cudaSuccess ||
       cudaMalloc((void**)&b->d_rows, rows_bytes) != cudaSuccess || cudaMalloc((void**)&b->d_status, 16) != cudaSuccess) {
     batch_free_persistent(b);
     return bfail(b, SWCS_ERR_OOM, "batch: device memory for the persistent launch");
   }
   b->rows_bytes = rows_bytes;
   b->nblocks = nblocks;
-  if (cudaMemcpy(b->d_inst, hi.data(), n * sizeof(BatchInst), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(b->d_sched0, hs.data(), n * sizeof(BatchSched), cudaMemcpyHostToDevice) != cudaSuccess)
+  b->n_kernel = nk;
+  if (cudaMemcpy(b->d_inst, hi.data(), nk * sizeof(BatchInst), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(b->d_sched0, hs.data(), nk * sizeof(BatchSched), cudaMemcpyHostToDevice) != cudaSuccess)
     return bfail(b, SWCS_ERR_CUDA, "batch: descriptor upload failed");
   const uint64_t timeout = b->timeout_ns;
   cudaError_t e = cudaStreamBeginCapture(b->origin, cudaStreamCaptureModeRelaxed);
   if (e != cudaSuccess) return bfail(b, SWCS_ERR_CUDA, std::string("begin capture: ") + cudaGetErrorString(e));
-  cudaMemcpyAsync(b->d_sched, b->d_sched0, n * sizeof(BatchSched), cudaMemcpyDeviceToDevice, b->origin);
+  cudaEventRecord(b->fork, b->origin);
+  // the gates that are launches of their own, each instance on its stream
+  int status = SWCS_OK;
+  for (int i = 0; i < n && !status; ++i) {
+    if (!own[i]) continue;
+    swcs_ctx* c = b->inst[i];
+    cudaStreamWaitEvent(c->st, b->fork, 0);
+    GateRun run;
+    run.one_cluster = true;
+    status = run_gates(c, (const uint8_t*)c->ops_dev.p, (const double*)c->cs_dev.p, b->n_ops[i], b->n_keep[i], true, run);
+    if (status) bfail(b, status, "batch capture: " + c->err);
+    cudaEventRecord(b->done[i], c->st);
+  }
   cudaMemsetAsync(b->d_status, 0, 16, b->origin);
-  cudaMemsetAsync(b->d_rows, 0, rows_bytes, b->origin);
-  e = launch_batch((const BatchInst*)b->d_inst, b->d_sched, n, b->d_rows, row_stride, b->d_status, nblocks, dyn, timeout,
-                   b->origin);
+  if (b->d_nmat) cudaMemsetAsync(b->d_nmat, 0, n * sizeof(long long), b->origin);  // stays 0 where an instance stops early
+  if (nk) {
+    cudaMemcpyAsync(b->d_sched, b->d_sched0, nk * sizeof(BatchSched), cudaMemcpyDeviceToDevice, b->origin);
+    cudaMemsetAsync(b->d_rows, 0, rows_bytes, b->origin);
+    e = launch_batch((const BatchInst*)b->d_inst, b->d_sched, nk, b->d_rows, row_stride, b->d_status, nblocks, dyn, timeout,
+                     b->origin);
+  }
+  cudaEventRecord(b->fork, b->origin);  // from here on: after the kernel
+  // the chains: an instance follows its gates and the instance before it, those with the shortest gates first
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::sort(order.begin(), order.end(), [&](int x, int y) {
+    const double gx = (double)b->n_ops[x] * b->max_state[x], gy = (double)b->n_ops[y] * b->max_state[y];
+    return own[x] != own[y] ? own[x] > own[y] : gx < gy;
+  });
+  for (int l = 0; l < kBatchLanes && e == cudaSuccess && !status; ++l) {
+    int first = -1;
+    for (int i : order) {
+      if (lane[i] != l || status) continue;
+      if (first < 0) first = i;
+      const cudaStream_t ls = b->streams[first];
+      cudaStreamWaitEvent(ls, own[i] ? b->done[i] : b->fork, 0);
+      swcs_ctx* c = b->inst[i];
+      const cudaStream_t st = c->st;
+      c->st = ls;
+      status = enqueue_density(c, (double*)c->gdev.p, b->max_state[i], own[i] ? nullptr : b->d_nmat + i, b->lane_mem[l],
+                               b->lane_mem[l] + rdm_gamma_doubles(c->n / 2));
+      c->st = st;
+      if (status) bfail(b, status, "batch capture: " + c->err);
+    }
+    if (first < 0) continue;
+    cudaEventRecord(b->done[first], b->streams[first]);
+    cudaStreamWaitEvent(b->origin, b->done[first], 0);
+  }
   cudaGraph_t g = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(b->origin, &g);
+  if (status) {
+    if (g) cudaGraphDestroy(g);
+    return status;
+  }
   if (e != cudaSuccess || e2 != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
     return bfail(b, SWCS_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
@@ -2211,7 +2376,7 @@ int batch_check(swcs_batch* b) {
     if (cudaMemcpy(st, b->d_status, 8, cudaMemcpyDeviceToHost) != cudaSuccess)
       return bfail(b, SWCS_ERR_CUDA, "batch run: status read failed");
     if (st[1] != 0) return bfail(b, SWCS_ERR_TIMEOUT, "batch run: a bounded wait for work ran out");
-    if (st[0] != (int)b->inst.size()) return bfail(b, SWCS_ERR_CUDA, "batch run: not every instance finished");
+    if (st[0] != b->n_kernel) return bfail(b, SWCS_ERR_CUDA, "batch run: not every instance finished");
   }
   for (swcs_ctx* c : b->inst) {
     int r = check_device(c, "batch instance");

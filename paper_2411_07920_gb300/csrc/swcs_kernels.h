@@ -226,6 +226,7 @@ struct BatchInst {
   double* g;           // pool gradient [pool_size]
   int64_t pool_size;
   double* eout;        // E, <psi|psi>
+  long long* n_mat;    // the sweep goes through the density matrices after this kernel: takes the state's size
 };
 
 // One published phase of an instance (two slots, by parity of the phase number).
