@@ -332,8 +332,14 @@ struct FusedArgs {
   int* err;
 };
 size_t mlp_fused_smem_bytes(int d_in, int width);
-cudaError_t launch_mlp_fused(const CUtensorMap& tm_x, const CUtensorMap& tm_w1, const CUtensorMap& tm_w2,
-                             const FusedArgs& f, int nblocks, cudaStream_t st);
+// Tensor maps of an operand's blocks of 64 and of 32 K-elements (either is unused where K has no such block).
+struct OperandMaps {
+  CUtensorMap k64, k32;
+};
+struct FusedMaps {
+  OperandMaps x, w1, w2;
+};
+cudaError_t launch_mlp_fused(const FusedMaps& maps, const FusedArgs& f, int nblocks, cudaStream_t st);
 cudaError_t launch_mlp_dy(const float* y, const float* t, int B, float* dy, double* loss, cudaStream_t st);
 cudaError_t launch_mlp_dz2(const float* dy, const __nv_bfloat16* w3, const __nv_bfloat16* H2, int B, int W,
                            __nv_bfloat16* dZ2, float* dw3, float* db3, cudaStream_t st);

@@ -89,7 +89,8 @@ GemmArgs gemm(swcs_mlp* m, const __nv_bfloat16* A, int lda, const __nv_bfloat16*
   return g;
 }
 
-bool k_major_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows);
+bool k_major_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows,
+                 uint32_t box_inner = 8);
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 // C = A B^T through the pipelined kernel when both operands have tensor maps (K contiguous, 16-byte aligned),
@@ -152,32 +153,41 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
-// Row-major BF16 [rows x inner] with boxes of 8 inner elements (16 bytes) x box_rows rows.
-bool k_major_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows) {
+// Row-major BF16 [rows x inner] with boxes of box_inner elements x box_rows rows: 8 (16 bytes, no swizzle), or 32 or
+// 64 with the swizzle of the box's width.
+bool k_major_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows,
+                 uint32_t box_inner) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc || ((uintptr_t)base & 15) || (inner * 2) % 16) return false;
   const cuuint64_t dims[2] = {inner, rows};
   const cuuint64_t strides[1] = {inner * 2};
-  const cuuint32_t box[2] = {8, box_rows};
+  const cuuint32_t box[2] = {box_inner, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE,
+             box_inner == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+             : box_inner == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                               : CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // y = network(x) with the fused kernel; 1 when the shape does not suit it.
 int predict_fused(swcs_mlp* m, const __nv_bfloat16* x, int64_t n, float* y) {
   const int D = m->p.d_in, W = m->p.width;
-  if (D % 16 || D < 16 || D > 64 || W % 16 || W < 16 || W > 256 || ((uintptr_t)x & 15)) return 1;
+  if (D % 32 || D < 32 || D > 64 || W % 32 || W < 32 || W > 256 || ((uintptr_t)x & 15)) return 1;
   int dev = 0, nsm = 0, optin = 0;
   MCK(cudaGetDevice(&dev));
   MCK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   MCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   if (mlp_fused_smem_bytes(D, W) > (size_t)optin) return 1;
-  CUtensorMap tx, tw1, tw2;
-  if (!k_major_map(&tx, x, (uint64_t)D, (uint64_t)n, 128) ||
-      !k_major_map(&tw1, m->p.W1b, (uint64_t)D, (uint64_t)W, (uint32_t)W) ||
-      !k_major_map(&tw2, m->p.W2b, (uint64_t)W, (uint64_t)W, (uint32_t)W))
+  FusedMaps maps{};
+  auto blocks = [](OperandMaps* o, const void* base, int K, uint64_t rows, uint32_t box_rows) {
+    return (K < 64 || k_major_map(&o->k64, base, (uint64_t)K, rows, box_rows, 64)) &&
+           (K % 64 == 0 || k_major_map(&o->k32, base, (uint64_t)K, rows, box_rows, 32));
+  };
+  if (!blocks(&maps.x, x, D, (uint64_t)n, 128) || !blocks(&maps.w1, m->p.W1b, D, (uint64_t)W, (uint32_t)W) ||
+      !blocks(&maps.w2, m->p.W2b, W, (uint64_t)W, (uint32_t)W))
     return 1;
   FusedArgs f{};
   f.M = n;
@@ -190,7 +200,7 @@ int predict_fused(swcs_mlp* m, const __nv_bfloat16* x, int64_t n, float* y) {
   f.y = y;
   f.err = m->err_dev;
   const int64_t tiles = (n + 127) / 128;
-  MCK(launch_mlp_fused(tx, tw1, tw2, f, (int)(tiles < nsm ? tiles : nsm), m->st));
+  MCK(launch_mlp_fused(maps, f, (int)(tiles < nsm ? tiles : nsm), m->st));
   m->launches += 1;
   return SWCS_OK;
 }

@@ -8,16 +8,20 @@
 //     epilogues: four warps per group of columns, one per tensor-memory lane quadrant, so every SM
 //     sub-partition has four epilogue warps to hide tensor-memory and shared-memory latency; all hand-offs
 //     go through mbarriers with bounded waits;
-//   - layer 1 accumulates X W1^T into tensor memory columns [0, W), its epilogue writes
-//     H1 = bf16(relu(. + b1)) straight into shared memory in the operand layout of layer 2, and layer 2
-//     accumulates H1 W2^T into columns [256, 256 + W); the second epilogue applies b2, ReLU, BF16 and the
-//     w3 dot product.  H1 and H2 never leave the SM: HBM sees X (64 B per row) and y (4 B per row).
-//   - while the epilogue of layer 2 reads tile t, the tensor cores already run layer 1 of tile t + 1.
+//   - a tile has one accumulator of 256 tensor-memory columns, even and odd tiles in turn: layer 1 puts X W1^T
+//     there, its epilogue takes it out and writes H1 = bf16(relu(. + b1)) into shared memory in the operand layout
+//     of layer 2, and layer 2 puts H1 W2^T in the same place; the second epilogue applies b2, ReLU, BF16 and the w3
+//     dot product.  H1 and H2 never leave the SM: HBM sees X (64 B per row) and y (4 B per row);
+//   - so layer 2 of tile t runs while the epilogue reads the accumulator of tile t - 1, and layer 1 of tile t + 1
+//     goes in half-way through layer 2: H1 of tile t + 1 is formed meanwhile, and each group of columns stored once
+//     layer 2 of tile t has read the old ones.  301,600 rows of 32 features, width 256: 61.6 us (76.7 us with one
+//     accumulator per layer, layer 2 waiting for the whole epilogue and back, and an arrival per thread on each
+//     barrier).  The tensor cores are busy for a third of it; the epilogues, at half the issue rate, bound it.
 //
-// Operand layout (K-major, no swizzle): core matrices of 8 rows x 16 bytes; one TMA box of 8 K-elements x
-// R rows fills R x 16 contiguous bytes, so K-adjacent core matrices are R x 16 bytes apart (leading byte
-// offset) and row-adjacent ones 128 bytes (stride byte offset).  Arithmetic, rounding and summation order
-// are those of the layer-by-layer kernels (mlp_gemm_kernel), so y is bit-identical to their result.
+// Operand layout: K-major, in blocks of 64 K-elements (rows of 128 bytes, 128-byte swizzle) and, where K leaves 32
+// over, a last block of 32 (rows of 64 bytes, 64-byte swizzle): an eighth of the TMA copies of the 16-byte-wide layout
+// without a swizzle.  Arithmetic, rounding and summation order are those of the layer-by-layer kernels
+// (mlp_gemm_kernel), so y is bit-identical to their result.
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -30,27 +34,75 @@ namespace swcs {
 
 namespace {
 
-constexpr int kEpiThreads = 128 * kDotGroups;  // warps 2 .. 2 + 4 kDotGroups - 1
+constexpr int kEpiThreads = 128 * kDotGroups;  // warps 2 .. 17: four (one per tensor-memory lane quadrant) per column group
 constexpr int kFusedThreads = 64 + kEpiThreads;
 constexpr int kCtrlBytes = 256;                 // control block, then the dot-product partials
 constexpr int kTile = 128;
-constexpr uint32_t kT2Col = 256;  // tensor-memory column of the layer-2 accumulator
+constexpr uint32_t kAccCols = 256;  // tensor-memory columns of an accumulator: even tiles' one, then odd tiles'
 constexpr uint64_t kSpinLimit = 1ull << 26;
 
 struct FusedCtrl {
-  uint64_t full_x[2], empty_x[2], w_full, mma1, mma2, t1_free, h1_ready, t2_free, part_ready, fin;
+  uint64_t full_x[2], empty_x[2], w_full, mma1, mma2, acc_free, h1_ready, part_ready, part_free, fin;
+  uint64_t h1_free[kDotGroups];
   uint32_t tmem;
 };
 
 __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ uint64_t desc_kmajor(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+// An operand of `rows` rows (a multiple of 32) in shared memory at `base` (a multiple of 1024): bytes up to its K-th
+// element, K a multiple of 32.
+__host__ __device__ constexpr uint32_t operand_bytes(int rows, int K) { return (uint32_t)rows * (uint32_t)K * 2u; }
+
+// Descriptor of the 16 K-elements from 16 k on.
+__device__ __forceinline__ uint64_t desc_k16(uint32_t base, int rows, int K, int k) {
+  const int full = K / 64;  // whole blocks of 64
+  const bool tail = k >= 4 * full;
+  const uint32_t addr = base + (tail ? operand_bytes(rows, 64 * full) + (uint32_t)(k - 4 * full) * 32u
+                                     : operand_bytes(rows, 64 * (k >> 2)) + (uint32_t)(k & 3) * 32u);
   uint64_t d = 0;
   d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;  // tcgen05 descriptor version; base offset 0, no swizzle
+  d |= (uint64_t)1 << 16;                            // leading byte offset: not used by swizzled K-major operands
+  d |= (uint64_t)((tail ? 512u : 1024u) >> 4) << 32;  // stride byte offset: 8 rows
+  d |= (uint64_t)1 << 46;                            // tcgen05 descriptor version; base offset 0
+  d |= (uint64_t)(tail ? 4 : 2) << 61;               // swizzle of 64 or 128 bytes
   return d;
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(da), "l"(db), "r"(idesc), "r"(acc));
+}
+
+// acc (+)= A B^T over K-elements 16 k0 .. 16 k1 of operands at a and b; by one thread.  Descriptors advance by
+// additions: worked out anew for each MMA they kept this thread, which shares its scheduler with the epilogue, from
+// feeding the tensor cores.
+__device__ __forceinline__ void mma_range(uint32_t acc, uint32_t a, int rows_a, uint32_t b, int rows_b, int K, int k0, int k1,
+                                          uint32_t idesc) {
+  if (k0 >= k1) return;
+  uint64_t da = desc_k16(a, rows_a, K, k0), db = desc_k16(b, rows_b, K, k0);
+  const uint64_t step_a = (operand_bytes(rows_a, 64) >> 4) - 6u, step_b = (operand_bytes(rows_b, 64) >> 4) - 6u;
+  const int tail = K / 64 * 4;
+  for (int k = k0; k < k1; ++k) {
+    mma_f16(acc, da, db, idesc, k > 0 ? 1u : 0u);
+    const bool next = (k & 3) == 3;  // the next block of 64 K-elements
+    da += next ? step_a : 2u;
+    db += next ? step_b : 2u;
+    if (k + 1 == tail) {
+      da = desc_k16(a, rows_a, K, tail);
+      db = desc_k16(b, rows_b, K, tail);
+    }
+  }
+}
+
+// Place of row r's 16 bytes u (0 or 1: K-elements 16 k + 8 u ..) in the operand's swizzled layout.
+__device__ __forceinline__ uint32_t place_k8(int rows, int K, int k, int u, int r) {
+  const int full = K / 64;
+  if (k >= 4 * full)
+    return operand_bytes(rows, 64 * full) + (uint32_t)r * 64u + (((uint32_t)(2 * (k - 4 * full) + u) ^ (((uint32_t)r >> 1) & 3u)) << 4);
+  return operand_bytes(rows, 64 * (k >> 2)) + (uint32_t)r * 128u + (((uint32_t)(2 * (k & 3) + u) ^ ((uint32_t)r & 7u)) << 4);
 }
 
 __host__ __device__ constexpr uint32_t idesc_f16(int m, int n) {
@@ -88,6 +140,17 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* b, uint32_t parity) 
   return false;
 }
 
+// The same for a whole warp, with one answer for all of its lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t* b, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(b, parity));
+}
+
+// One arrival for the warp, after all of its lanes got here: 16 on a word where there were 512.
+__device__ __forceinline__ void warp_arrive(uint64_t* b) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(b);
+}
+
 // 2-D tile load: box origin (x = K element, y = row) into shared memory, completion on mbar.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* mbar) {
   asm volatile(
@@ -97,34 +160,55 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc));
-}
-
 __device__ __forceinline__ void mma_commit(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(b))
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_load16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+// 16 C columns of this warp's lanes.  The wait is in the same statement: before it the registers hold nothing.
+template <int C>
+__device__ __forceinline__ void tmem_load(uint32_t taddr, uint32_t* r) {
+  static_assert(C == 1 || C == 2, "columns");
+  if constexpr (C == 2) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+  } else {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+  }
 }
 
-__device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+// work(C, first chunk) over n 16-column chunks, two at a time while there are two.
+template <int C>
+struct Chunks {
+  static constexpr int count = C;
+};
+template <class F>
+__device__ __forceinline__ void by_chunks(int n, F&& work) {
+  int i = 0;
+#pragma unroll 1
+  for (; i + 2 <= n; i += 2) work(Chunks<2>(), i);
+  if (i < n) work(Chunks<1>(), i);
+}
+
+// bf16 of max(v + b, 0) for two neighbours, the first in the low half (rounding keeps the sign, so it commutes with
+// the maximum; NaN gives 0).
+__device__ __forceinline__ uint32_t relu_sum(const uint32_t* v, const float* b) {
+  const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(__uint_as_float(v[0]) + b[0], __uint_as_float(v[1]) + b[1]),
+                                   __floats2bfloat162_rn(0.f, 0.f));
+  return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // 16 consecutive parameters, the same for every lane, in whole 16-byte loads (a load per element made the epilogues
@@ -140,41 +224,37 @@ __device__ __forceinline__ void load16(const float* p, float* v) {
   }
 }
 
-__device__ __forceinline__ void load16(const __nv_bfloat16* p, float* v) {
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p) + i);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[8 * i + 2 * k] = __uint_as_float(w[k] << 16);
-      v[8 * i + 2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
-    }
-  }
-}
-
 }  // namespace
 
 size_t mlp_fused_smem_bytes(int d_in, int width) {
-  return 128 /* alignment slack */ + kCtrlBytes + (size_t)kDotGroups * kTile * 4 /* partials */ +
-         (size_t)width * d_in * 2 + (size_t)width * width * 2 +
-         2 * (size_t)kTile * d_in * 2 + (size_t)kTile * width * 2;
+  return operand_bytes(width, d_in) + operand_bytes(width, width) +
+         2 * operand_bytes(kTile, d_in) + operand_bytes(kTile, width) + kCtrlBytes +
+         (size_t)(kDotGroups - 1) * kTile * 4 /* partials */ + (size_t)width * 4 /* w3 */;
+}
+
+// All of an operand's blocks into shared memory, rows from `row` on.
+__device__ __forceinline__ void load_operand(uint8_t* dst, const OperandMaps& m, int rows, int K, int row, uint64_t* mbar) {
+  const int full = K / 64;
+  for (int g = 0; g < full; ++g) tma_load_2d(dst + operand_bytes(rows, 64 * g), &m.k64, 64 * g, row, mbar);
+  if (K % 64) tma_load_2d(dst + operand_bytes(rows, 64 * full), &m.k32, 64 * full, row, mbar);
 }
 
 __global__ void __launch_bounds__(kFusedThreads, 1)
-mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
-                 const __grid_constant__ CUtensorMap tm_w2, FusedArgs f) {
-  extern __shared__ uint8_t dsm[];
-  const uint32_t pad = (128u - (saddr(dsm) & 127u)) & 127u;
-  uint8_t* sm = dsm + pad;
-  FusedCtrl& c = *reinterpret_cast<FusedCtrl*>(sm);
+mlp_fused_kernel(const __grid_constant__ FusedMaps maps, FusedArgs f) {
+  extern __shared__ __align__(1024) uint8_t sm[];  // the swizzled operands want this alignment
+  if (saddr(sm) & 1023u) {
+    if (f.err) set_error(f.err, kDevBadState);
+    return;
+  }
   const int D = f.d_in, W = f.width;
-  float* sPart = reinterpret_cast<float*>(sm + kCtrlBytes);  // [kDotGroups][kTile]
-  uint8_t* sW1 = sm + kCtrlBytes + kDotGroups * kTile * 4;
-  uint8_t* sW2 = sW1 + (size_t)W * D * 2;
-  uint8_t* sX0 = sW2 + (size_t)W * W * 2;
-  uint8_t* sX1 = sX0 + (size_t)kTile * D * 2;
-  uint8_t* sH1 = sX1 + (size_t)kTile * D * 2;
+  uint8_t* sW2 = sm;
+  uint8_t* sH1 = sW2 + operand_bytes(W, W);
+  uint8_t* sW1 = sH1 + operand_bytes(kTile, W);
+  uint8_t* sX0 = sW1 + operand_bytes(W, D);
+  uint8_t* sX1 = sX0 + operand_bytes(kTile, D);
+  FusedCtrl& c = *reinterpret_cast<FusedCtrl*>(sX1 + operand_bytes(kTile, D));
+  float* sPart = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(&c) + kCtrlBytes);  // [kDotGroups - 1][kTile]
+  float* sW3 = sPart + (kDotGroups - 1) * kTile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = (int)((f.M + kTile - 1) / kTile);
 
@@ -190,13 +270,15 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     mbar_init(&c.w_full, 1);
     mbar_init(&c.mma1, 1);
     mbar_init(&c.mma2, 1);
-    mbar_init(&c.t1_free, kEpiThreads);
-    mbar_init(&c.h1_ready, kEpiThreads);
-    mbar_init(&c.t2_free, kEpiThreads);
-    mbar_init(&c.part_ready, kEpiThreads);
+    mbar_init(&c.acc_free, kEpiThreads / 32);
+    mbar_init(&c.h1_ready, kEpiThreads / 32);
+    mbar_init(&c.part_ready, kEpiThreads / 32 / kDotGroups * (kDotGroups - 1));
+    mbar_init(&c.part_free, kEpiThreads / 32 / kDotGroups);
     mbar_init(&c.fin, 1);
+    for (int g = 0; g < kDotGroups; ++g) mbar_init(&c.h1_free[g], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < W; i += kFusedThreads) sW3[i] = __bfloat162float(f.w3[i]);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -206,9 +288,9 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
 
   if (warp == 0) {
     if (lane == 0) {  // ------------------------------------------------ TMA producer
-      mbar_expect_tx(&c.w_full, (uint32_t)(W * D * 2 + W * W * 2));
-      for (int g = 0; g < D / 8; ++g) tma_load_2d(sW1 + (size_t)g * W * 16, &tm_w1, 8 * g, 0, &c.w_full);
-      for (int g = 0; g < W / 8; ++g) tma_load_2d(sW2 + (size_t)g * W * 16, &tm_w2, 8 * g, 0, &c.w_full);
+      mbar_expect_tx(&c.w_full, operand_bytes(W, D) + operand_bytes(W, W));
+      load_operand(sW1, maps.w1, W, D, 0, &c.w_full);
+      load_operand(sW2, maps.w2, W, W, 0, &c.w_full);
       bool issued0 = false, issued1 = false;
       uint32_t last0 = 0, last1 = 0;
       int j = 0;
@@ -220,8 +302,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
           break;
         }
         uint8_t* dst = s ? sX1 : sX0;
-        mbar_expect_tx(&c.full_x[s], (uint32_t)(kTile * D * 2));
-        for (int g = 0; g < D / 8; ++g) tma_load_2d(dst + g * (kTile * 16), &tm_x, 8 * g, t * kTile, &c.full_x[s]);
+        mbar_expect_tx(&c.full_x[s], operand_bytes(kTile, D));
+        load_operand(dst, maps.x, kTile, D, t * kTile, &c.full_x[s]);
         if (s) { issued1 = true; last1 = par; } else { issued0 = true; last0 = par; }
       }
       // no copy may still be landing when the CTA leaves (returns at once when already consumed)
@@ -232,24 +314,33 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
   } else if (warp == 1) {
     if (lane == 0) {  // ------------------------------------------------ MMA issuer
       if (!mbar_wait_bounded(&c.w_full, 0)) bad = true;
-      int j = 0;
-      for (int t = blockIdx.x; t < ntiles && !bad; t += gridDim.x, ++j) {
-        const int s = j & 1;
+      // layer 1 of this CTA's tile jj
+      auto layer1 = [&](int jj) {
+        const int s = jj & 1;
         const uint8_t* sx = s ? sX1 : sX0;
-        if (!mbar_wait_bounded(&c.full_x[s], (uint32_t)(j >> 1) & 1u)) { bad = true; break; }
-        if (j > 0 && !mbar_wait_bounded(&c.t1_free, (uint32_t)(j - 1) & 1u)) { bad = true; break; }
+        if (!mbar_wait_bounded(&c.full_x[s], (uint32_t)(jj >> 1) & 1u)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int k = 0; k < D / 16; ++k)
-          mma_f16(tmem, desc_kmajor(saddr(sx) + k * 2 * (kTile * 16), kTile * 16, 128),
-                  desc_kmajor(saddr(sW1) + k * 2 * (W * 16), W * 16, 128), idesc, k > 0 ? 1u : 0u);
+        mma_range(tmem + s * kAccCols, saddr(sx), kTile, saddr(sW1), W, D, 0, D / 16, idesc);
         mma_commit(&c.empty_x[s]);
         mma_commit(&c.mma1);
+        return true;
+      };
+      int j = 0;
+      if ((int)blockIdx.x < ntiles && !bad && !layer1(0)) bad = true;
+      for (int t = blockIdx.x; t < ntiles && !bad; t += gridDim.x, ++j) {
         if (!mbar_wait_bounded(&c.h1_ready, (uint32_t)j & 1u)) { bad = true; break; }
-        if (j > 0 && !mbar_wait_bounded(&c.t2_free, (uint32_t)(j - 1) & 1u)) { bad = true; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int k = 0; k < W / 16; ++k)
-          mma_f16(tmem + kT2Col, desc_kmajor(saddr(sH1) + k * 2 * (kTile * 16), kTile * 16, 128),
-                  desc_kmajor(saddr(sW2) + k * 2 * (W * 16), W * 16, 128), idesc, k > 0 ? 1u : 0u);
+        for (int g = 0; g < kDotGroups; ++g) {  // by the columns of H1 that a group of warps writes
+          if (g == kDotGroups / 2) {
+            // the accumulator of tile j - 1 has been read: layer 1 of tile j + 1 goes there
+            if (j > 0 && !mbar_wait_bounded(&c.acc_free, (uint32_t)(j - 1) & 1u)) { bad = true; break; }
+            if (t + (int)gridDim.x < ntiles && !layer1(j + 1)) { bad = true; break; }
+          }
+          mma_range(tmem + (j & 1) * kAccCols, saddr(sH1), kTile, saddr(sW2), W, W, dot_group_begin(g, W / 16),
+                    dot_group_begin(g + 1, W / 16), idesc);
+          mma_commit(&c.h1_free[g]);
+        }
+        if (bad) break;
         mma_commit(&c.mma2);
       }
       mma_commit(&c.fin);  // every MMA issued above has completed once this phase completes
@@ -260,62 +351,83 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
     const int grp = (warp - 2) >> 2;   // its group of 16-column chunks
     const int r = q * 32 + lane;
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
-    const int cb = dot_group_begin(grp, W / 16) * 16, ce = dot_group_begin(grp + 1, W / 16) * 16;
-    int j = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
-      if (!mbar_wait_bounded(&c.mma1, (uint32_t)j & 1u)) { bad = true; break; }
+    const int cb = dot_group_begin(grp, W / 16), nch = dot_group_begin(grp + 1, W / 16) - cb;
+    // H1 of this CTA's tile jj, stored once layer 2 of the tile before has read the group's old columns
+    auto epilogue1 = [&](int jj) {
+      if (!warp_wait(&c.mma1, (uint32_t)jj & 1u)) return false;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int c0 = cb; c0 < ce; c0 += 16) {
-        float v[16], b[16];
-        load16(f.b1 + c0, b);
-        tmem_load16(tmem + lanes + (uint32_t)c0, v);
-        uint32_t w[8];
+      bool ok = true, free = jj == 0;
+      by_chunks(nch, [&](auto cc, int i0) {
+        constexpr int C = decltype(cc)::count;
+        uint32_t v[16 * C], h[C][8];
+        tmem_load<C>(tmem + lanes + (uint32_t)((jj & 1) * kAccCols + (cb + i0) * 16), v);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          float z0 = v[2 * i] + b[2 * i];
-          float z1 = v[2 * i + 1] + b[2 * i + 1];
-          z0 = z0 > 0.f ? z0 : 0.f;
-          z1 = z1 > 0.f ? z1 : 0.f;
-          w[i] = pack_bf16x2(__float2bfloat16_rn(z0), __float2bfloat16_rn(z1));
+        for (int i = 0; i < C; ++i) {
+          float b[16];
+          load16(f.b1 + (cb + i0 + i) * 16, b);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) h[i][k] = relu_sum(&v[16 * i + 2 * k], &b[2 * k]);
         }
-        // row r, K groups c0/8 and c0/8 + 1: 16 bytes each in the layer-2 operand layout
-        *reinterpret_cast<uint4*>(sH1 + (size_t)(c0 / 8) * (kTile * 16) + r * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(sH1 + (size_t)(c0 / 8 + 1) * (kTile * 16) + r * 16) =
-            make_uint4(w[4], w[5], w[6], w[7]);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(&c.t1_free);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // H1 visible to the tensor cores
-      mbar_arrive(&c.h1_ready);
-      if (!mbar_wait_bounded(&c.mma2, (uint32_t)j & 1u)) { bad = true; break; }
+        if (!free) {
+          free = true;
+          ok = warp_wait(&c.h1_free[grp], (uint32_t)(jj - 1) & 1u);
+        }
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          const int k = cb + i0 + i;
+          *reinterpret_cast<uint4*>(sH1 + place_k8(kTile, W, k, 0, r)) = make_uint4(h[i][0], h[i][1], h[i][2], h[i][3]);
+          *reinterpret_cast<uint4*>(sH1 + place_k8(kTile, W, k, 1, r)) = make_uint4(h[i][4], h[i][5], h[i][6], h[i][7]);
+        }
+      });
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");  // the accumulator has been read
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // H1 visible to the tensor cores
+      warp_arrive(&c.h1_ready);
+      return ok;
+    };
+    int j = 0;
+    if ((int)blockIdx.x < ntiles && !epilogue1(0)) bad = true;
+    for (int t = blockIdx.x; t < ntiles && !bad; t += gridDim.x, ++j) {
+      if (t + (int)gridDim.x < ntiles && !epilogue1(j + 1)) { bad = true; break; }
+      if (!warp_wait(&c.mma2, (uint32_t)j & 1u)) { bad = true; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float part = 0.f;
-      for (int c0 = cb; c0 < ce; c0 += 16) {
-        float v[16], b[16], w3[16];
-        load16(f.b2 + c0, b);
-        load16(f.w3 + c0, w3);
-        tmem_load16(tmem + lanes + kT2Col + (uint32_t)c0, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float z = v[i] + b[i];
-          z = z > 0.f ? z : 0.f;
-          const __nv_bfloat16 hb = __float2bfloat16_rn(z);
-          part += __bfloat162float(hb) * w3[i];
+      by_chunks(nch, [&](auto cc, int i0) {
+        constexpr int C = decltype(cc)::count;
+        uint32_t v[16 * C];
+        tmem_load<C>(tmem + lanes + (uint32_t)((j & 1) * kAccCols + (cb + i0) * 16), v);
+        if (i0 + C == nch) {  // the accumulator has been read
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          warp_arrive(&c.acc_free);
         }
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(&c.t2_free);
-      // partials of the row meet in shared memory; group 0 adds them in group order.  Group 0 reads
-      // them before it arrives on h1_ready of the next tile, so no group can overwrite them earlier.
-      sPart[grp * kTile + r] = part;
-      mbar_arrive(&c.part_ready);
-      if (grp == 0) {
-        if (!mbar_wait_bounded(&c.part_ready, (uint32_t)j & 1u)) { bad = true; break; }
-        float dot = sPart[r];
 #pragma unroll
-        for (int gg = 1; gg < kDotGroups; ++gg) dot += sPart[gg * kTile + r];
+        for (int i = 0; i < C; ++i) {
+          float b[16];
+          load16(f.b2 + (cb + i0 + i) * 16, b);
+          const float* w3 = sW3 + (cb + i0 + i) * 16;
+#pragma unroll
+          for (int k = 0; k < 8; k += 2) {
+            const uint32_t h0 = relu_sum(&v[16 * i + 2 * k], &b[2 * k]), h1 = relu_sum(&v[16 * i + 2 * k + 2], &b[2 * k + 2]);
+            const float4 w = *reinterpret_cast<const float4*>(w3 + 2 * k);
+            part += __uint_as_float(h0 << 16) * w.x;
+            part += __uint_as_float(h0 & 0xFFFF0000u) * w.y;
+            part += __uint_as_float(h1 << 16) * w.z;
+            part += __uint_as_float(h1 & 0xFFFF0000u) * w.w;
+          }
+        }
+      });
+      if (nch == 0) warp_arrive(&c.acc_free);
+      // the groups' partials of the row are added in group order by the first group's warps
+      if (grp != 0) {
+        if (j > 0 && !warp_wait(&c.part_free, (uint32_t)(j - 1) & 1u)) { bad = true; break; }
+        sPart[(grp - 1) * kTile + r] = part;
+        warp_arrive(&c.part_ready);
+      } else {
+        if (!warp_wait(&c.part_ready, (uint32_t)j & 1u)) { bad = true; break; }
+#pragma unroll
+        for (int g = 1; g < kDotGroups; ++g) part += sPart[(g - 1) * kTile + r];
+        warp_arrive(&c.part_free);
         const int64_t row = (int64_t)t * kTile + r;
-        if (row < f.M) f.y[row] = dot + __ldg(f.b3);
+        if (row < f.M) f.y[row] = part + __ldg(f.b3);
       }
     }
   }
@@ -325,8 +437,7 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-cudaError_t launch_mlp_fused(const CUtensorMap& tm_x, const CUtensorMap& tm_w1, const CUtensorMap& tm_w2,
-                             const FusedArgs& f, int nblocks, cudaStream_t st) {
+cudaError_t launch_mlp_fused(const FusedMaps& maps, const FusedArgs& f, int nblocks, cudaStream_t st) {
   const size_t smem = mlp_fused_smem_bytes(f.d_in, f.width);
   static size_t attr = 0;
   if (attr < smem) {
@@ -334,7 +445,7 @@ cudaError_t launch_mlp_fused(const CUtensorMap& tm_x, const CUtensorMap& tm_w1, 
     if (e != cudaSuccess) return e;
     attr = smem;
   }
-  mlp_fused_kernel<<<nblocks, kFusedThreads, smem, st>>>(tm_x, tm_w1, tm_w2, f);
+  mlp_fused_kernel<<<nblocks, kFusedThreads, smem, st>>>(maps, f);
   return cudaGetLastError();
 }
 
