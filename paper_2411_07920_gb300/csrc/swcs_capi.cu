@@ -883,12 +883,14 @@ int energy_rows(swcs_ctx* c, double* sig_out) {
     if (nd <= kMaxPairDets) {
       PairArgs a;
       const int r = pair_args(c, nd, true, &a);
-      if (r) return r;
-      a.sig = sig_out;
-      CK(launch_k(c, kKEnergy, [&] { return launch_pairs_energy(a, nd, c->nsm, c->st); }));
-      c->launches += 3;
-      CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(ctrl(c)->acc, ctrl(c)->eout, c->st); }));
-      return SWCS_OK;
+      if (r && r != SWCS_ERR_OOM) return r;
+      if (!r) {
+        a.sig = sig_out;
+        CK(launch_k(c, kKEnergy, [&] { return launch_pairs_energy(a, nd, c->nsm, c->st); }));
+        c->launches += 3;
+        CK(launch_k(c, kKOther, [&] { return launch_finalize_energy(ctrl(c)->acc, ctrl(c)->eout, c->st); }));
+        return SWCS_OK;
+      }
     }
   }
   return sweep_rows(c, nullptr, -1, true, nullptr, true, sig_out);
@@ -967,8 +969,9 @@ int sweep_density(swcs_ctx* c, double* d_g, int64_t nd) {
   if (ensure(c, c->rdm_gamma, rdm_gamma_doubles(m) * 8) || ensure(c, c->rdm_work, rdm_work_doubles(m) * 8) ||
       ensure(c, c->rdm_tab, rdm_table_doubles(m) * 8))
     return 1;
-  const int r = ensure_rdm_tables(c);
-  return r ? r : enqueue_density(c, d_g, nd, nullptr, (double*)c->rdm_gamma.p, (double*)c->rdm_work.p);
+  int r = ensure_rdm_tables(c);
+  if (!r) r = enqueue_density(c, d_g, nd, nullptr, (double*)c->rdm_gamma.p, (double*)c->rdm_work.p);
+  return r == SWCS_ERR_OOM ? 1 : r;
 }
 
 int sweep(swcs_ctx* c, double* d_g, const uint32_t* sel = nullptr) {
@@ -1543,9 +1546,22 @@ static int copy_out_sorted(swcs_ctx* c, const double* vals, int64_t n, uint64_t*
   int r;
   DevBuf* kb[2] = {&c->sort_k1, &c->sort_k2};
   DevBuf* vb[2] = {&c->sort_v1, &c->sort_v2};
-  for (int i = 0; i < 2; ++i)
-    if ((r = ensure(c, *kb[i], (size_t)n * 8)) || (r = ensure(c, *vb[i], (size_t)n * 8))) return r;
-  if ((r = ensure(c, c->sort_cnt, sort_count_words(n) * 4))) return r;
+  bool room = ensure(c, c->sort_cnt, sort_count_words(n) * 4) == SWCS_OK;
+  for (int i = 0; i < 2 && room; ++i)
+    room = ensure(c, *kb[i], (size_t)n * 8) == SWCS_OK && ensure(c, *vb[i], (size_t)n * 8) == SWCS_OK;
+  if (!room) {  // no memory for the sort on the device
+    CK(cudaMemcpyAsync(h_keys, c->keys_a.p, 8 * n, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaMemcpyAsync(h_vals, vals, 8 * n, cudaMemcpyDeviceToHost, c->st));
+    if ((r = check_device(c, where))) return r;
+    std::vector<std::pair<uint64_t, double>> v(n);
+    for (int64_t i = 0; i < n; ++i) v[i] = {h_keys[i], h_vals[i]};
+    std::sort(v.begin(), v.end(), [](const auto& x, const auto& y) { return x.first < y.first; });
+    for (int64_t i = 0; i < n; ++i) {
+      h_keys[i] = v[i].first;
+      h_vals[i] = v[i].second;
+    }
+    return SWCS_OK;
+  }
   bool second = false;
   CK(launch_k(c, kKOther, [&] {
     return launch_sort_pairs((const uint64_t*)c->keys_a.p, vals, (uint64_t*)kb[0]->p, (double*)vb[0]->p, (uint64_t*)kb[1]->p,
