@@ -340,19 +340,23 @@ def run_swcs(args):
     ctx.profile_enable(False)
     ms_per_step, value = aggregate(total_ms, args.steps, world, dev)
 
-    # hash probes of one more (untimed) step: lookups and the index slots they visit, per second of the
-    # kernels that make them (gate kernel: partner lookups of the merge; row sweep: neighbour discovery)
+    # hash probes of one more (untimed) step: lookups and the index slots they visit, per second of the kernels that
+    # make them (gate kernel: partner lookups of the merge; row sweep: neighbour discovery).  Counting sends the pool
+    # sweep through the alpha-string rows.
     ctx.set_option("count_probes", 1)
     ctx.probe_counts(reset=True)
+    ctx.profile_enable(True)
     step()
     pc = ctx.probe_counts(reset=True)
+    counted = ctx.profile_read(reset=True)
+    ctx.profile_enable(False)
     ctx.set_option("count_probes", 0)
-    g_ms = prof.get("ansatz", (0.0, 0))[0] / max(args.steps, 1)
-    r_ms = prof.get("row_sweep", (0.0, 0))[0] / max(args.steps, 1)
+    g_ms = counted.get("ansatz", (0.0, 0))[0]
+    r_ms = counted.get("row_sweep", (0.0, 0))[0]
     probes = {"gate": {"lookups": pc["gate_lookups"], "slots": pc["gate_slots"],
                        "slots_per_lookup": round(pc["gate_slots"] / max(pc["gate_lookups"], 1), 4),
                        "lookups_per_s": pc["gate_lookups"] / (g_ms / 1e3) if g_ms > 0 else None},
-              "row_sweep": {"lookups": pc["row_lookups"], "slots": pc["row_slots"],
+              "row_sweep": {"lookups": pc["row_lookups"], "slots": pc["row_slots"], "ms": round(r_ms, 3),
                             "slots_per_lookup": round(pc["row_slots"] / max(pc["row_lookups"], 1), 4),
                             "lookups_per_s": pc["row_lookups"] / (r_ms / 1e3) if r_ms > 0 else None}}
 
@@ -366,51 +370,62 @@ def run_swcs(args):
     dom_ms, dom_n = kinds[dom]
     buckets = max(stats["ext_buckets"], 1)
     pairs = n_det * (n_conn + 1)
-    # algorithmic bytes per connected (D, E) pair: the scatter reads the key and
-    # sigma_E and writes sigma_E (24 B), the gather reads them (16 B); the row
-    # sweep does both in one launch
-    per_pair = {"sigma_scatter": 24.0, "pool_gather": 16.0, "row_sweep": 40.0}
     peaks = {}
     try:
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
     except Exception:
         pass
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
-    if dom == "row_sweep":
-        bytes_per_launch = per_pair[dom] * pairs
-    elif dom in per_pair:
-        bytes_per_launch = per_pair[dom] * pairs / buckets
-    elif dom == "ansatz":
-        # per gate: read S (16 B/det), write and re-read Phi (32 B), select reads (8 B/pass), write S (16 B)
-        bytes_per_launch = (16 + 32 + 8 * max(stats["select_passes"] / max(stats["gates"], 1), 1) + 16) * \
-            stats["gate_dets"] / max(dom_n, 1)
-    else:
-        bytes_per_launch = 16.0 * pairs
-    achieved = bytes_per_launch / (dom_ms / dom_n / 1e3) / 1e9
-    roof = {"kernel": dom, "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
-            "frac": achieved / hbm_peak, "traffic": measured_traffic(dom, args),
-            "peak_source": "measured" if "hbm_gbs" in peaks else "fallback"}
-    gate_ms = prof.get("ansatz", (0.0, 0))[0]
+    # the pool sweep went through the density matrices of the state (it reports neither buckets nor row clusters)
+    density = stats["ext_buckets"] == 0 and prof.get("row_sweep", (0.0, 0))[1] > 0
+    m = w.n_so // 2
+    mix, tri = m * (m * (m - 1) // 2), math.comb(m, 3)
+
+    def kernel_bytes(kind, launches_of_kind):
+        """Bytes one launch of a kind cannot do without."""
+        if kind == "row_sweep" and density:
+            return 8.0 * 2 * (mix * mix + tri * tri)  # each three-body matrix read once
+        # per connected (D, E) pair: the scatter reads the key and sigma_E and writes sigma_E (24 B), the gather
+        # reads them (16 B); the row sweep does both in one launch
+        if kind == "row_sweep":
+            return 40.0 * pairs
+        if kind in ("sigma_scatter", "pool_gather"):
+            return (24.0 if kind == "sigma_scatter" else 16.0) * pairs / buckets
+        if kind == "ansatz":
+            # per gate and determinant: key and amplitude read, amplitude written; a general select pass reads the
+            # amplitudes again
+            return (24 + 8 * stats["select_passes"] / max(stats["gates"], 1)) * stats["gate_dets"] / launches_of_kind
+        return 16.0 * n_det
+
+    def hbm_roofline(kind, ms, n):
+        b = kernel_bytes(kind, n)
+        ach = b / (ms / n / 1e3) / 1e9
+        return {"kernel": kind, "bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
+                "frac": ach / hbm_peak, "bytes_per_launch": b,
+                "traffic": measured_traffic("density" if kind == "row_sweep" and density else kind, args),
+                "peak_source": "measured" if "hbm_gbs" in peaks else "fallback"}
+    roof = hbm_roofline(dom, dom_ms, dom_n)
+    if dom == "row_sweep" and density:
+        # bound by the FP64 pipe, not by HBM: FP64 operations of the captured launch (their number follows from the
+        # state) against the nominal rate of two FMA per clock and SM
+        flops = measured_flops("density", args)
+        roof["kernel"] = "density-matrix contraction"
+        if flops is not None:
+            fp64_peak = 2 * 2 * torch.cuda.get_device_properties(dev).multi_processor_count * 2.07
+            ach = flops / (dom_ms / dom_n / 1e3) / 1e9
+            roof.update({"bound": "fp64", "achieved": ach, "peak": fp64_peak, "unit": "GFLOP/s",
+                         "frac": ach / fp64_peak, "flops_per_launch": flops, "peak_source": "nominal"})
+    gate_ms, gate_n = prof.get("ansatz", (0.0, 0))
     gate_dets_per_s = stats["gate_dets"] / (gate_ms / 1e3) if gate_ms > 0 else None
-    # the other two kernels of the path, on the same measured peak
+    # the other kernels of the path, on the same measured peak
     rooflines = {}
-    gate_n = prof.get("ansatz", (0.0, 0))[1]
     if gate_ms > 0 and gate_n > 0:
-        # per gate: read S (16 B/det), write and re-read Phi (32 B), select reads (8 B/pass), write S' (16 B),
-        # with |Phi| and |S'| taken as |S|
-        passes = stats["select_passes"] / max(stats["gates"], 1)
-        gb = (16 + 32 + 8 * passes + 16) * stats["gate_dets"] / gate_n
-        ach = gb / (gate_ms / gate_n / 1e3) / 1e9
-        rooflines["gate"] = {"kernel": "ansatz", "bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
-                             "frac": ach / hbm_peak, "bytes_per_launch": gb, "select_passes_per_gate": passes,
-                             "traffic": measured_traffic("ansatz", args)}
+        rooflines["gate"] = hbm_roofline("ansatz", gate_ms, gate_n)
+        rooflines["gate"]["select_passes_per_gate"] = stats["select_passes"] / max(stats["gates"], 1)
     if energy_ms:
-        # energy <psi|H|psi>: 16 B (key and amplitude) per connection of every determinant probed in the
-        # state, the bytes of the probe formulation (the row kernel in energy-only mode reads fewer)
-        eb = 16.0 * n_det * (n_conn + 1)
-        ach = eb / (min(energy_ms) / 1e3) / 1e9
-        rooflines["energy"] = {"kernel": "row_sweep (energy only)", "bound": "hbm", "achieved": ach, "peak": hbm_peak,
-                               "unit": "GB/s", "frac": ach / hbm_peak, "bytes_per_launch": eb, "traffic": None}
+        # energy <psi|H|psi> from the pairs of determinants inside the state: reads the state (16 B each); bound by
+        # the string comparisons and lookups in L2, not by these bytes
+        rooflines["energy"] = hbm_roofline("energy", min(energy_ms), 1)
     launches = int(stats["kernel_launches"])
 
     # ------------------------------------------------------------ end to end through the host API
@@ -512,7 +527,9 @@ TRAFFIC_FILES = {
     "row_sweep": ("profiles/row_sweep_so52_e12_N1e6.md",
                   ["paper_2411_07920_gb300/csrc/swcs_rowsweep.cu", "paper_2411_07920_gb300/csrc/swcs_rowsweep.cuh"]),
     "ansatz": ("profiles/ansatz_so52_e12_N1e6.md",
-               ["paper_2411_07920_gb300/csrc/swcs_ansatz.cu", "paper_2411_07920_gb300/csrc/swcs_select.cuh"]),
+               ["paper_2411_07920_gb300/csrc/swcs_gates.cu", "paper_2411_07920_gb300/csrc/swcs_select.cuh"]),
+    "density": ("profiles/density_so52_e12_N1e6.md",
+                ["paper_2411_07920_gb300/csrc/swcs_rdm.cu", "paper_2411_07920_gb300/csrc/swcs_pairs.cu"]),
 }
 
 
@@ -525,10 +542,10 @@ def source_sha16(paths):
     return h.hexdigest()[:16]
 
 
-def measured_traffic(kernel, args):
-    """DRAM bytes per launch of the dominant kernel from its committed ncu summary,
-    only for the workload and launch shape that were captured and while the
-    kernel's source is the one that was captured (else None)."""
+def committed_figure(kernel, args, key):
+    """A whole number per launch from a kernel's committed ncu summary, only for
+    the workload and launch shape that were captured and while the kernel's
+    source is the one that was captured (else None)."""
     if kernel not in TRAFFIC_FILES:
         return None
     if args.sweep == 1 or any(getattr(args, k) != v for k, v in TRAFFIC_CAPTURED.items()):
@@ -537,11 +554,21 @@ def measured_traffic(kernel, args):
     try:
         text = open(os.path.join(ROOT, summary)).read()
         want = text.split("source_sha256:")[1].split()[0]
-        traffic = int(text.split("traffic_bytes_per_launch:")[1].split()[0])
+        value = int(text.split(key)[1].split()[0])
         have = source_sha16(srcs)
     except (OSError, IndexError, ValueError):
         return None
-    return traffic if have == want else None
+    return value if have == want else None
+
+
+def measured_traffic(kernel, args):
+    """DRAM bytes per launch."""
+    return committed_figure(kernel, args, "traffic_bytes_per_launch:")
+
+
+def measured_flops(kernel, args):
+    """FP64 operations per launch (an FMA counts two)."""
+    return committed_figure(kernel, args, "fp64_ops_per_launch:")
 
 
 def run_screen_leg(swcs, ctx, w, args, torch, frac=0.05):

@@ -373,6 +373,10 @@ int swcs_pool_screen_dev(swcs_ctx* ctx, swcs_mlp* m, double frac, int64_t* d_sub
  * that finishes a phase's last tile runs its epilogue and publishes the next
  * phase.  Waits for work are bounded (SWCS_ERR_TIMEOUT).  The launch is
  * captured in a CUDA graph together with the reset of its scheduler words.
+ * Instances whose pool sweep is faster through the density matrices (the
+ * rule of swcs_pool_gradients, at their bound on the state) get that sweep as
+ * launches of their own in the same graph, and up to 131,072 determinants
+ * their gates too, beside the kernel.
  * Mode 1 instead captures each instance's own kernels on a branch of a graph.
  *   swcs_batch_add     copies the inputs (same meaning as swcs_load_hamiltonian
  *                      and swcs_apply_ansatz); *index_out = instance index
