@@ -711,7 +711,7 @@ def run_configs_leg(swcs, I, torch, reps=5):
 
 def run_batch_leg(swcs, I, torch, n_inst=64, seed0=100, reps=3):
     """64 uneven instances (n_so in U{16..40}, n_e in U{4..12}, 20-150 gates,
-    N_keep log-uniform 1e3-1e5): one persistent launch for all of them
+    N_keep log-uniform 1e3-1e5): one graph launch for all of them
     (autotuned, settings cached in JSON) against the same per-instance kernels
     launched back to back on one stream, and against the host API called
     instance by instance; every instance's result checked against its own
@@ -768,7 +768,8 @@ def run_batch_leg(swcs, I, torch, n_inst=64, seed0=100, reps=3):
     for c in ctxs:
         c.close()
     b.close()
-    return {"instances": n_inst, "launch": "one persistent kernel, (instance, phase, tile) work items",
+    return {"instances": n_inst, "launch": "one graph: a persistent kernel of (instance, phase, tile) work items, large instances by "
+                                             "cluster gates and density-matrix sweeps beside it",
             "launch_ms": round(1e3 * t_launch, 3), "back_to_back_ms": round(1e3 * t_back, 3),
             "host_api_ms": round(1e3 * min(th), 3), "speedup_vs_back_to_back": round(t_back / t_launch, 3),
             "speedup_vs_host_api": round(min(th) / t_launch, 3), "max_abs_diff_all_instances": err,
